@@ -81,6 +81,11 @@ struct Table {
     float2* data = nullptr;               // C-1, complex float32
     int store = WG_F32;                   // samples the gridder reads
     void* data_lp = nullptr;              // C-1 as complex bf16 / f16 (store != WG_F32)
+    // C-1 as the gridder and the degridder read it: sample pairs {re, re', im, im'} (pairs.cuh)
+    float4* pairs = nullptr;
+    void* pairs_lp = nullptr;             // the same as bf16 / f16 (store != WG_F32)
+    unsigned* poffsets_d = nullptr;       // [K] first pair of each plane
+    int64_t n_pairs = 0;
     double* zeta = nullptr;               // C-3 [K beta^2]
     int* supports_d = nullptr;            // C-2 supports [K]
     int* offsets_d = nullptr;             // C-2 offsets [K]

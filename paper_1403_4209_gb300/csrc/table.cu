@@ -145,6 +145,42 @@ static int default_nk(int s_max)
     return n;
 }
 
+// C-1 as pairs (pairs.cuh): plane k (blockIdx.y), per sub-kernel H = (S + 1) / 2 rows of S pairs; pair
+// (i, c) holds the samples of rows i and i + H in column c (zero past the last row).
+__global__ void k_table_pairs(const float2* __restrict__ src, const int* __restrict__ supports,
+                              const int* __restrict__ offsets, const unsigned* __restrict__ poffsets, int beta2, int store,
+                              void* __restrict__ dst)
+{
+    const int k = blockIdx.y, S = supports[k], H = (S + 1) / 2;
+    const float2* s = src + offsets[k];
+    const int64_t total = (int64_t)beta2 * S * H;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t sub = i / (S * H);
+        const int r = (int)(i - sub * (S * H));
+        const float2* p = s + sub * S * S + r;
+        const float2 a = p[0];
+        const float2 b = r + H * S < S * S ? p[H * S] : make_float2(0.f, 0.f);
+        const int64_t o = (int64_t)poffsets[k] + i;
+        if (store == WG_F32) {
+            reinterpret_cast<float4*>(dst)[o] = make_float4(a.x, b.x, a.y, b.y);
+        } else if (store == WG_BF16) {
+            reinterpret_cast<__nv_bfloat162*>(dst)[2 * o] = __floats2bfloat162_rn(a.x, b.x);
+            reinterpret_cast<__nv_bfloat162*>(dst)[2 * o + 1] = __floats2bfloat162_rn(a.y, b.y);
+        } else {
+            reinterpret_cast<__half2*>(dst)[2 * o] = __floats2half2_rn(a.x, b.x);
+            reinterpret_cast<__half2*>(dst)[2 * o + 1] = __floats2half2_rn(a.y, b.y);
+        }
+    }
+}
+
+static int fill_pairs(const Table& t, int store, void* dst, cudaStream_t s)
+{
+    k_table_pairs<<<dim3(num_sms(), t.K), 256, 0, s>>>(t.data, t.supports_d, t.offsets_d, t.poffsets_d, t.beta * t.beta,
+                                                      store, dst);
+    WG_LAUNCHED("k_table_pairs");
+    return WG_OK;
+}
+
 __global__ void k_table_lp(const float2* __restrict__ src, int64_t n, int store, void* __restrict__ dst)
 {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -160,16 +196,22 @@ int set_table_store(Table& t, int store)
 {
     if (store != WG_F32 && store != WG_BF16 && store != WG_F16) return fail(WG_E_INVALID_ARG, "unknown store dtype %d", store);
     cudaFree(t.data_lp);
+    cudaFree(t.pairs_lp);
     t.data_lp = nullptr;
+    t.pairs_lp = nullptr;
     t.store = WG_F32;
     if (store == WG_F32) return WG_OK;
-    if (cudaMalloc(&t.data_lp, 4 * (size_t)std::max<int64_t>(t.n_samples, 1)) != cudaSuccess) {
+    if (cudaMalloc(&t.data_lp, 4 * (size_t)std::max<int64_t>(t.n_samples, 1)) != cudaSuccess ||
+        cudaMalloc(&t.pairs_lp, 8 * (size_t)std::max<int64_t>(t.n_pairs, 1)) != cudaSuccess) {
         cudaGetLastError();
+        cudaFree(t.data_lp);
+        t.data_lp = nullptr;
         return fail(WG_E_OOM, "cannot allocate the low-precision table");
     }
     if (t.n_samples > 0) {
         k_table_lp<<<(unsigned)((t.n_samples + 255) / 256), 256>>>(t.data, t.n_samples, store, t.data_lp);
         WG_LAUNCHED("k_table_lp");
+        if (int rc = fill_pairs(t, store, t.pairs_lp, nullptr)) return rc;
     }
     WG_CUDA(cudaDeviceSynchronize());
     t.store = store;
@@ -180,6 +222,12 @@ int free_table(Table& t)
 {
     cudaFree(t.data_lp);
     t.data_lp = nullptr;
+    cudaFree(t.pairs_lp);
+    cudaFree(t.pairs);
+    cudaFree(t.poffsets_d);
+    t.pairs_lp = nullptr;
+    t.pairs = nullptr;
+    t.poffsets_d = nullptr;
     cudaFree(t.data);
     cudaFree(t.zeta);
     cudaFree(t.supports_d);
@@ -199,17 +247,23 @@ int free_table(Table& t)
 static int finish_layout(Table& t)
 {
     t.offsets.resize(t.K);
-    int64_t off = 0;
+    int64_t off = 0, poff = 0;
+    std::vector<unsigned> poffsets(t.K);
     t.max_support = 0;
     for (int k = 0; k < t.K; ++k) {
         t.offsets[k] = (int)off;
+        poffsets[k] = (unsigned)poff;              // at most one pair a sample: below 2^31
+        poff += (int64_t)t.beta * t.beta * t.supports[k] * ((t.supports[k] + 1) / 2);
         off += (int64_t)t.beta * t.beta * t.supports[k] * t.supports[k];
         t.max_support = std::max(t.max_support, t.supports[k]);
     }
     if (off >= (int64_t)1 << 31) return fail(WG_E_OOB_SUPPORT, "kernel table has %lld samples (limit 2^31)", (long long)off);
     t.n_samples = off;
+    t.n_pairs = poff;
     if (cudaMalloc(&t.data, sizeof(float2) * std::max<int64_t>(off, 1)) != cudaSuccess ||
         cudaMalloc(&t.zeta, sizeof(double) * t.K * t.beta * t.beta) != cudaSuccess ||
+        cudaMalloc(&t.pairs, sizeof(float4) * std::max<int64_t>(poff, 1)) != cudaSuccess ||
+        cudaMalloc(&t.poffsets_d, sizeof(unsigned) * t.K) != cudaSuccess ||
         cudaMalloc(&t.supports_d, sizeof(int) * t.K) != cudaSuccess ||
         cudaMalloc(&t.offsets_d, sizeof(int) * t.K) != cudaSuccess ||
         cudaMalloc(&t.wbounds_d, sizeof(double) * t.K) != cudaSuccess ||
@@ -221,6 +275,7 @@ static int finish_layout(Table& t)
     }
     WG_CUDA(cudaMemcpy(t.supports_d, t.supports.data(), sizeof(int) * t.K, cudaMemcpyHostToDevice));
     WG_CUDA(cudaMemcpy(t.offsets_d, t.offsets.data(), sizeof(int) * t.K, cudaMemcpyHostToDevice));
+    WG_CUDA(cudaMemcpy(t.poffsets_d, poffsets.data(), sizeof(unsigned) * t.K, cudaMemcpyHostToDevice));
     // nearest plane in sqrt(w): plane k is chosen when b_k <= w < b_{k+1}, with
     // b_m = w_max (t t), t = (m - 1/2) / (K - 1), m = 1..K (b_K bounds the last plane)
     std::vector<double> wb(t.K, 0.0);
@@ -345,6 +400,7 @@ int build_table(const wg_table_desc& d, Table& t, cudaStream_t s)
             k_zeta_f32<<<(nz + 255) / 256, 256, 0, s>>>(t.zeta, nz, t.zeta_f);
             count_launch();
         }
+        if ((rc = fill_pairs(t, WG_F32, t.pairs, s)) != WG_OK) break;
         cudaError_t e = cudaStreamSynchronize(s);
         if (e != cudaSuccess) rc = cuda_fail(e, "conv_table_build");
     } while (0);
@@ -382,7 +438,10 @@ int import_table(int K, int beta, double w_max, double du, int s0, const int* su
         free_table(t);
         return fail(WG_E_CUDA, "table upload failed");
     }
-    return WG_OK;
+    int rc2 = fill_pairs(t, WG_F32, t.pairs, nullptr);
+    if (rc2 == WG_OK && cudaDeviceSynchronize() != cudaSuccess) rc2 = cuda_fail(cudaGetLastError(), "k_table_pairs");
+    if (rc2 != WG_OK) free_table(t);
+    return rc2;
 }
 
 }  // namespace wg
