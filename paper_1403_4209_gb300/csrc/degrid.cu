@@ -288,9 +288,10 @@ __device__ __forceinline__ bool entry_ok(const int4& E, const int* __restrict__ 
 // acc[0 .. n_entries * 2P) = 0
 __global__ void k_degrid_zero(float4* __restrict__ acc, const long long* __restrict__ scal, int P)
 {
-    const long long n4 = scal[0] * P / 2;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n4; i += (long long)gridDim.x * blockDim.x)
-        acc[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    const long long n2 = scal[0] * P, n4 = n2 / 2;
+    const long long i0 = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    for (long long i = i0; i < n4; i += (long long)gridDim.x * blockDim.x) acc[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (i0 == 0 && (n2 & 1)) reinterpret_cast<float2*>(acc)[n2 - 1] = make_float2(0.f, 0.f);
 }
 
 template <int P, int RT>

@@ -128,3 +128,18 @@ def test_nonfinite_visibilities_stay_in_their_footprints(P, comp):
     pl0 = oracle.place(batch.uvw.cpu().numpy(), batch.freq.cpu().numpy(), 1.0, N, ref, flag=fl)
     want = oracle.grid_plain(pl0, ref, vis, wt, fl, N)[0, ..., 0]
     assert np.abs(g[..., 0][~hit] - want[~hit]).max() < 1e-5 * np.abs(want).max()
+
+
+def test_degridding_again_with_an_odd_number_of_entries():
+    # the per-entry sums start at zero in every call, also the last entry's when the list's length is
+    # odd at one polarisation
+    supports, P, N = [9], 1, 64
+    ref, tab, pl, batch, vis, wt, fl = _case(supports, P, N, 300, 3)
+    g = wg.Grid(N, 1.0, P, 1)
+    work = wg.WorkList(300, 1, P)
+    for rows in (299, 300):              # one of the two lists has an odd length
+        b = wg.VisBatch(batch.uvw[:rows], batch.freq, batch.vis[:rows], batch.weight[:rows], batch.flag[:rows])
+        wg.vis_compress(g, tab, b, work, compress=False)
+        g.data.fill_(1.0)
+        first = wg.degrid_vis(g, tab, b, work).clone()
+        assert torch.equal(wg.degrid_vis(g, tab, b, work), first)
