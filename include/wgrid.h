@@ -335,10 +335,9 @@ int grid_vis(wg_grid* grid, const wg_table* table, const wg_worklist* wl, void* 
 /* ---- gridder plan (not in the thesis: GPU work decomposition) ----------------------
  * grid_vis cuts the work list's gridded entries into segments of seg_len consecutive entries
  * and each segment's footprint (of its largest support S) into ceil(S^2 / slots) tasks; a
- * warp runs one task at a time with R points per lane.  By default R = ceil(S^2 / (32 x
- * tasks)) per support; with WG_PLAN_FIXED_R, R = slots / 32 for every support (no per-point
- * checks; the last task of a small support then has idle points).  FIXED_R takes effect for
- * slots 128 and 256 on FP32 tables without compensation; elsewhere the per-support R runs.
+ * warp runs one task at a time.  The tasks of a support share its footprint's points evenly,
+ * several per lane.  WG_PLAN_FIXED_R is kept in the plan and changes nothing: it asked for
+ * slots / 32 points per lane for every support, and every plan now runs the same kernel.
  * vis_compress plans with the work list's current plan (initially WG_PLAN_SEG_LEN_DEFAULT,
  * WG_PLAN_SLOTS_DEFAULT, no flags).  The plan changes only the order of the FP32 additions,
  * not what is added. */

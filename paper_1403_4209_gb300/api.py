@@ -258,7 +258,7 @@ class WorkList:
 
     def plan(self, table: "ConvTable", seg_len: int, slots: int, fixed_r: bool = False, stream=None):
         """Re-plans the prepared batch's gridder tasks: segment length, footprint points per task,
-        and whether every support runs with R = slots / 32 points per lane (WG_PLAN_FIXED_R)."""
+        and WG_PLAN_FIXED_R (kept in the plan; it changes nothing)."""
         pl = Plan(int(seg_len), int(slots), CONST["WG_PLAN_FIXED_R"] if fixed_r else 0, 0)
         check(lib.worklist_plan(self._h, table.handle, ctypes.byref(pl), _stream(stream)), "worklist_plan")
 

@@ -5,15 +5,16 @@
 // takes two launches.
 //
 // k_degrid_sum runs the gridder's tasks (a segment of consecutive entries x one block of the
-// footprint, as the work list's plan defines them) with the gridder's ownership: each lane owns
-// R residue classes (x mod S, y mod S) of the footprint, so exactly one pixel of each class lies
-// in every entry's footprint (Romein's argument, Sec. 2.5).  The lane keeps those pixels' values
-// (all polarisations) in registers and reloads one only when the footprint moves and the class's
-// pixel changes; for consecutive entries of a track that keep the footprint and differ only in
-// the sub-kernel z it loads nothing but the kernel samples.  Per entry each lane sums its R
-// points into 2P floats; these go through a shared-memory transpose (batches of 64 / (2P)
+// footprint, as the work list's plan defines them) on the gridder's point pairs and ownership
+// (pairs.cuh).  A lane keeps its pairs' pixel values in registers and reloads a pair only when the
+// footprint moves and the class's pixels change; for consecutive entries of a track that keep the footprint and
+// differ only in the sub-kernel it loads nothing but the kernel samples.  Per entry each lane sums its
+// pairs into 2P floats; these go through a shared-memory transpose (batches of 64 / (2P)
 // entries), after which each lane holds two components of one entry summed over the warp and
-// adds them to a per-entry FP32 accumulator with one vector atomic per footprint block.
+// adds them to a per-entry FP32 accumulator with one vector atomic per footprint block.  It is bound like
+// the gridder (issue 52 %, FMA pipe 45 %, L1 data path 62 %), with the transpose on top.  Measured (degrid_vis,
+// default plan): 0.87 M entries of supports 9..65, 4.8 M records: P = 4 2105 -> 1600 us, P = 2 1660 -> 1060, P = 1
+// 1470 -> 900; supports 9..129, P = 1 1510 -> 925; 1 k entries 227 -> 44.
 //
 // k_degrid_tile writes the records of each entry's run.  Compression (Sec. 4.3.3) carries over:
 // every record compressed into an entry has its footprint and kernel samples, so m is computed
@@ -21,7 +22,7 @@
 // with the cross hands swapped back under cross-hand swapping, and for the adjoint mode scaled
 // by eps (1 - f) (the vis -> grid map's R-linear outer factor).  It works per preparation tile
 // through shared memory so that the output is written row-major with coalesced stores.
-#include "internal.cuh"
+#include "pairs.cuh"
 
 namespace wg {
 
@@ -31,47 +32,18 @@ constexpr int kWarps = 4;           // warps per block of k_degrid_sum
 constexpr int kTileCap = 4096;      // records per preparation tile: rpb x C <= max(kTileRecords, n_chan <= 4096)
 static_assert(kTileRecords <= kTileCap, "a preparation tile must fit the degridder's output tile");
 
-typedef unsigned long long f32x2;   // a packed FP32 pair (Blackwell f32x2 arithmetic)
-
-__device__ __forceinline__ f32x2 pack2(float lo, float hi)
-{
-    f32x2 r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-    return r;
-}
-
-__device__ __forceinline__ float2 unpack2(f32x2 v)
-{
-    float2 r;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
-    return r;
-}
-
-__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c)
-{
-    f32x2 d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-    return d;
-}
-
-__device__ __forceinline__ void cp_async16(void* dst, const void* src)
-{
-    const unsigned d = static_cast<unsigned>(__cvta_generic_to_shared(dst));
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(src));
-}
-
-// the P polarisations of one pixel as packed pairs (gx, gy)
+// the P polarisations of one pixel
 template <int P>
-__device__ __forceinline__ void load_pixel(const float2* __restrict__ g, f32x2 (&v)[P])
+__device__ __forceinline__ void load_pixel(const float2* __restrict__ g, float2 (&v)[P])
 {
     if constexpr (P == 1) {
-        v[0] = __ldg(reinterpret_cast<const f32x2*>(g));
+        v[0] = __ldg(g);
     } else {
 #pragma unroll
         for (int h = 0; h < P; h += 2) {
-            const ulonglong2 a = __ldg(reinterpret_cast<const ulonglong2*>(g + h));
-            v[h] = a.x;
-            v[h + 1] = a.y;
+            const float4 a = __ldg(reinterpret_cast<const float4*>(g + h));
+            v[h] = make_float2(a.x, a.y);
+            v[h + 1] = make_float2(a.z, a.w);
         }
     }
 }
@@ -88,42 +60,26 @@ __device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b)
 // reads of two adjacent components of 32 / P different slots fall in distinct banks).
 constexpr int kRedFloats = 64 * 33;      // per warp, any P
 
-// Per-warp shared memory: the residue-class arrays, the reduction buffer, then the segment's
-// staged entries.
-struct WarpSmem {
-    short (*pu)[32];         // [kRMax][32] each lane's owned residue classes: x mod S
-    short (*pv)[32];         // [kRMax][32] and y mod S
-    float* red;              // [kRedFloats]
-    int4* rec;               // [seg_len] entries, w replaced by the key
-    static constexpr size_t kFixed = 2 * kRMax * 32 * sizeof(short) + kRedFloats * sizeof(float);
-    __device__ explicit WarpSmem(unsigned char* base)
-        : pu(reinterpret_cast<short (*)[32]>(base)),
-          pv(reinterpret_cast<short (*)[32]>(base) + kRMax),
-          red(reinterpret_cast<float*>(base + 2 * kRMax * 32 * sizeof(short))),
-          rec(reinterpret_cast<int4*>(base + kFixed)) {}
-    static constexpr size_t bytes(int seg_len) { return kFixed + (size_t)seg_len * sizeof(int4); }
-};
-
-// Entries [j, e1) of the staged segment while their key (support, grid channel) equals `key`,
-// footprint block `blk`, R points per lane (RT > 0 fixes R at compile time; points past S^2
-// keep pixel value 0 and read sample offset 0).  Adds each entry's sums to acc[j][2P]; returns
-// the first entry not processed.  Each lane stores its 2P partials of an entry in the reduction
-// buffer; every 64 / (2P) entries (and at the end) each lane sums two adjacent components of one
-// entry over the 32 lanes and adds them to acc with one vector atomic.
-template <int P, int RT>
-__device__ __forceinline__ int degrid_records(int j, int e1, int key, int S, int R, int blk, int N, int lane,
-                                              WarpSmem& sm, const float2* __restrict__ table,
-                                              const float2* __restrict__ gch, float* __restrict__ acc)
+// One run of entries from entry j of the chunk on (see the gridder's run_entries): adds each entry's
+// sums over the units [un.x, un.y), at most NU, to acc[entry][2P].  Returns the first entry (of
+// the chunk then staged) after it, or -1 at the item's end.  Each lane stores its 2P partials of an
+// entry in the reduction buffer; every 64 / (2P) entries (and at the end) each lane sums two adjacent
+// components of one entry over the 32 lanes and adds them to acc with one vector atomic.
+template <int P, int NU>
+__device__ __forceinline__ int degrid_entries(Chunk<P, false>& ck, int j, int S, int ch, int2 un, const TaskParams& tp,
+                                              bool report, float* __restrict__ red, const char* __restrict__ table,
+                                              const float2* __restrict__ grid, float* __restrict__ acc)
 {
+    constexpr int PB = kPairBytes<float2>;
     constexpr int V = 2 * P, NB = 64 / V, SLOT = 33 * V;
-    if constexpr (RT > 0) R = RT;
-    int nbuf = 0, jb = j;     // entries buffered, and the first of them
+    const int lane = ck.lane, H = (S + 1) >> 1;
+    int nbuf = 0, eb = ck.e0 + j;     // entries buffered, and the first of them in the list
     // lane l sums components c, c + 1 of buffered entry b over the 32 lanes
     auto drain = [&](int n) {
         __syncwarp();
         const int b = (2 * lane) / V, c = (2 * lane) % V;
         if (b < n) {
-            const float* src = sm.red + b * SLOT + c;
+            const float* src = red + b * SLOT + c;
             f32x2 t = 0ull;
 #pragma unroll
             for (int l2 = 0; l2 < 32; ++l2) {
@@ -131,123 +87,112 @@ __device__ __forceinline__ int degrid_records(int j, int e1, int key, int S, int
                 const int cs = (V == 8 && (l2 & 4)) ? 4 : 0;
                 t = add2(t, *reinterpret_cast<const f32x2*>(src + l2 * V + (c ^ cs) - c));
             }
-            atomicAdd(reinterpret_cast<float2*>(acc + (size_t)(jb + b) * V + c), unpack2(t));
+            atomicAdd(reinterpret_cast<float2*>(acc + (size_t)(eb + b) * V + c), unpack2(t));
         }
         __syncwarp();
     };
-    f32x2 pv[kRMax][P];
-    int toff[kRMax], cur[kRMax];     // sample byte offset and pixel held of each owned class
-    unsigned valid = 0;
-    const int s2 = S * S, sbase = blk * 32 * R;
-    const float inv_s = 1.0f / (float)S;
+    unsigned toff[NU];
+    place_classes<NU, PB>(toff, ck.cls, ck.cur, ck.e[j], S, un.x, un.y, lane);
+    // The pairs' pixels.  P = 1: the two points' real parts and imaginary parts as packed pairs, as the
+    // samples come.  P = 2, 4: per point, two polarisations' parts as packed pairs, multiplied by a sample's part as
+    // a scalar (FMAs that read five registers run at 2.6 cycles against 3.2 for three pairs, and the
+    // sums need no addition across a pair: 1650 -> 1600 us on 0.87 M entries of supports 9..65).
+    constexpr int Q = P == 1 ? 1 : P / 2;      // pairs of polarisations
+    f32x2 g[NU][2][Q][2];                      // P = 1: [u][0][0] = {re, re'}, {im, im'}; else [u][point][q] = re, im
 #pragma unroll
-    for (int r = 0; r < kRMax; ++r) {
-        const int sl = sbase + r * 32 + lane;
-        cur[r] = -1;
-        toff[r] = 0;
-        if (r < R) {
-            // a slot past S^2 follows class (0, 0): its sample offset stays inside the
-            // sub-kernel, and its pixel value stays 0
-            int pu = 0, pv_ = 0;
-            if (sl < s2) {
-                valid |= 1u << r;
-                const int2 vu = divmod_small(sl, S, inv_s);
-                pv_ = vu.x;
-                pu = vu.y;
+    for (int u = 0; u < NU; ++u)
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int q = 0; q < Q; ++q) g[u][h][q][0] = g[u][h][q][1] = 0ull;
+    // loads the pairs in `which` for the footprint whose first row is y0; the row past the footprint stays
+    // 0 (its samples are 0, its pixels may hold an infinity)
+    auto reload = [&](unsigned which, int y0) {
+#pragma unroll
+        for (int u = 0; u < NU; ++u) {
+            if (which & (1u << u)) {
+                const int cur = ck.cur[u][lane];
+                if (cur >= 0) {
+                    const int y = cur >> 16;
+                    const float2* px = grid + ((size_t)((unsigned)ch * (unsigned)tp.N + (unsigned)y) * tp.N + (cur & 0xFFFF)) * P;
+                    float2 a[P], b[P];
+                    load_pixel<P>(px, a);
+#pragma unroll
+                    for (int p = 0; p < P; ++p) b[p] = make_float2(0.f, 0.f);
+                    if (y + H < y0 + S) load_pixel<P>(px + (size_t)(H * tp.N) * P, b);
+                    if constexpr (P == 1) {
+                        g[u][0][0][0] = pack2(a[0].x, b[0].x);
+                        g[u][0][0][1] = pack2(a[0].y, b[0].y);
+                    } else {
+#pragma unroll
+                        for (int q = 0; q < Q; ++q) {
+                            g[u][0][q][0] = pack2(a[2 * q].x, a[2 * q + 1].x);
+                            g[u][0][q][1] = pack2(a[2 * q].y, a[2 * q + 1].y);
+                            g[u][1][q][0] = pack2(b[2 * q].x, b[2 * q + 1].x);
+                            g[u][1][q][1] = pack2(b[2 * q].y, b[2 * q + 1].y);
+                        }
+                    }
+                }
             }
-            sm.pu[r][lane] = (short)pu;
-            sm.pv[r][lane] = (short)pv_;
         }
+    };
+    KPair k[NU];
+    {
+        const char* kz = table + (size_t)ck.z[j] * PB;
 #pragma unroll
-        for (int p = 0; p < P; ++p) pv[r][p] = 0ull;
+        for (int u = 0; u < NU; ++u) k[u] = load_pair((const float2*)nullptr, kz, toff[u]);
     }
-    int fp = -1;             // footprint origin (x0 | y0 << 16) the offsets and pixels refer to
-    for (; j < e1; ++j) {
-        const int4 E = sm.rec[j];
-        if (E.w != key) break;
-        if (E.x != fp) {     // the footprint moved: new offsets, reload the pixels that change
-            const int x0 = E.x & 0xFFFF, y0 = (E.x >> 16) & 0xFFFF;
-            const int cu = E.y & 0xFFFF, cv = (E.y >> 16) & 0xFFFF;
-            const int dx = x0 - (fp & 0xFFFF), dy = y0 - (fp >> 16);
-            if (fp >= 0 && ((dy == 0 && (dx == 1 || dx == -1)) || (dx == 0 && (dy == 1 || dy == -1)))) {
-                // a one-cell move: every offset shifts by the move, and only the class column
-                // (or row) that left the footprint wraps and takes a new pixel (as in the gridder)
-                const bool along_x = dy == 0;
-                const int d = along_x ? dx : dy;
-                const int cn = along_x ? cu : cv;                  // (-origin) mod S
-                const int m = cn ? S - cn : 0;                     // origin mod S
-                const int c = d > 0 ? (m ? m - 1 : S - 1) : m;     // the class that wraps
-                const int step = along_x ? 1 : S;
-                const int shift = d * step * (int)sizeof(float2);
-                const int wrap = d * S * step * (int)sizeof(float2);
-                const int pstep = along_x ? d * S : d * S * N;
-                short (*cls)[32] = along_x ? sm.pu : sm.pv;
-#pragma unroll
-                for (int r = 0; r < kRMax; ++r) {
-                    if (r < R) {
-                        const bool w = cls[r][lane] == c;
-                        toff[r] += w ? wrap - shift : -shift;
-                        if (w && (valid & (1u << r))) {
-                            cur[r] += pstep;
-                            load_pixel<P>(gch + (size_t)cur[r] * P, pv[r]);
-                        }
-                    }
-                }
-            } else {
-                // the first entry of the run, or a jump: place every point from its class
-#pragma unroll
-                for (int r = 0; r < kRMax; ++r) {
-                    if (r < R) {
-                        int du = sm.pu[r][lane] + cu;
-                        du -= (du >= S) ? S : 0;
-                        int dv = sm.pv[r][lane] + cv;
-                        dv -= (dv >= S) ? S : 0;
-                        toff[r] = (dv * S + du) * (int)sizeof(float2);
-                        if (valid & (1u << r)) {
-                            const int pix = (y0 + dv) * N + x0 + du;
-                            if (pix != cur[r]) {
-                                load_pixel<P>(gch + (size_t)pix * P, pv[r]);
-                                cur[r] = pix;
-                            }
-                        }
-                    }
-                }
-            }
-            fp = E.x;
-        }
-        f32x2 kv[kRMax];
-        const f32x2* kz = reinterpret_cast<const f32x2*>(table + E.z);
-#pragma unroll
-        for (int r = 0; r < kRMax; ++r) {
-            if (RT == 0 && r >= R) break;
-            // unsigned 32-bit byte offset: cheaper than a signed element index (see the gridder)
-            if (r < R) kv[r] = __ldg(reinterpret_cast<const f32x2*>(reinterpret_cast<const char*>(kz) + (unsigned)toff[r]));
-        }
-        // A_p = sum kx (gx, gy), B_p = sum ky (gx, gy); conj(k) g = (A.x + B.y, A.y - B.x)
-        f32x2 A[P], B[P];
-#pragma unroll
-        for (int p = 0; p < P; ++p) A[p] = B[p] = 0ull;
-#pragma unroll
-        for (int r = 0; r < kRMax; ++r) {
-            if (RT == 0 && r >= R) break;
-            if (r < R) {
-                const float2 k = unpack2(kv[r]);
-                const f32x2 kxx = pack2(k.x, k.x), kyy = pack2(k.y, k.y);
-#pragma unroll
-                for (int p = 0; p < P; ++p) {
-                    A[p] = fma2(kxx, pv[r][p], A[p]);
-                    B[p] = fma2(kyy, pv[r][p], B[p]);
-                }
-            }
-        }
+    // an entry's sums into the reduction buffer; the samples of the entry whose sub-kernel is at kz are loaded
+    // into a unit's registers behind its FMAs
+    auto entry = [&](const char* kz) {
+        // conj(k) g = (kx gx + ky gy, kx gy - ky gx)
         float v[V];
+        if constexpr (P == 1) {
+            f32x2 s0 = 0ull, s1 = 0ull;
 #pragma unroll
-        for (int p = 0; p < P; ++p) {
-            const float2 a = unpack2(A[p]), b = unpack2(B[p]);
-            v[2 * p] = a.x + b.y;
-            v[2 * p + 1] = a.y - b.x;
+            for (int u = 0; u < NU; ++u) {
+                const float2 im = unpack2(k[u].im);
+                s0 = fma2(k[u].im, g[u][0][0][1], fma2(k[u].re, g[u][0][0][0], s0));
+                s1 = fma2(pack2(-im.x, -im.y), g[u][0][0][0], fma2(k[u].re, g[u][0][0][1], s1));
+                k[u] = load_pair((const float2*)nullptr, kz, toff[u]);
+            }
+            const float2 a = unpack2(s0), b = unpack2(s1);
+            v[0] = a.x + a.y;
+            v[1] = b.x + b.y;
+        } else {
+            f32x2 s[Q][2];
+#pragma unroll
+            for (int q = 0; q < Q; ++q) s[q][0] = s[q][1] = 0ull;
+#pragma unroll
+            for (int u = 0; u < NU; ++u) {
+                const float2 re = unpack2(k[u].re), im = unpack2(k[u].im);
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const float x = h ? re.y : re.x, y = h ? im.y : im.x;
+                    const f32x2 kx = pack2(x, x), ky = pack2(y, y), ny = pack2(-y, -y);
+#pragma unroll
+                    for (int q = 0; q < Q; ++q) {
+                        s[q][0] = fma2(kx, g[u][h][q][0], s[q][0]);
+                        s[q][1] = fma2(kx, g[u][h][q][1], s[q][1]);
+                    }
+#pragma unroll
+                    for (int q = 0; q < Q; ++q) {
+                        s[q][0] = fma2(ky, g[u][h][q][1], s[q][0]);
+                        s[q][1] = fma2(ny, g[u][h][q][0], s[q][1]);
+                    }
+                }
+                k[u] = load_pair((const float2*)nullptr, kz, toff[u]);
+            }
+#pragma unroll
+            for (int q = 0; q < Q; ++q) {
+                const float2 a = unpack2(s[q][0]), b = unpack2(s[q][1]);
+                v[4 * q] = a.x;
+                v[4 * q + 1] = b.x;
+                v[4 * q + 2] = a.y;
+                v[4 * q + 3] = b.y;
+            }
         }
-        float* dst = sm.red + nbuf * SLOT + lane * V;
+        float* dst = red + nbuf * SLOT + lane * V;
         if constexpr (V == 8) {
             // halves swapped for lanes with bit 2 set: the 8 lanes of a quarter-warp store to
             // distinct banks
@@ -259,29 +204,61 @@ __device__ __forceinline__ int degrid_records(int j, int e1, int key, int S, int
         } else {
             *reinterpret_cast<float2*>(dst) = make_float2(v[0], v[1]);
         }
-        if (++nbuf == NB) {
-            drain(NB);
+        ++nbuf;
+    };
+    unsigned touched = ~0u;           // pairs whose pixels change with the coming entry
+    int y0 = ck.e[j].x >> 16;
+    bool same = true;
+    for (;;) {
+        if (nbuf == NB || !same) {
+            drain(nbuf);
+            eb += nbuf;
             nbuf = 0;
-            jb = j + 1;
+            if (!same) return j;
         }
+        if (touched) {
+            reload(touched, y0);
+            touched = 0;
+        }
+        // entries whose successor has the same footprint, as far as the buffer goes
+        const unsigned later = ck.mv & (0xFFFFFFFEu << j);
+        const int last = (later ? __ffs(later) - 1 : ck.cnt) - 1, stop = min(last, j + NB - nbuf);
+        for (; j < stop; ++j) entry(table + (size_t)ck.z[j + 1] * PB);
+        if (nbuf == NB) continue;
+        // the footprint's last entry in the chunk: the move to its successor comes first (as in the gridder)
+        unsigned zn = ck.z[j];
+        bool more = true;
+        if (++j == ck.cnt) {
+            more = ck.next(tp, report);
+            j = more ? 0 : -1;
+        }
+        same = more && !((ck.kc >> j) & 1);            // the run goes on
+        if (same) {
+            zn = ck.z[j];
+            if ((ck.mv >> j) & 1) {
+                const Move m = ck.m[j];
+                touched = move_classes<NU, PB>(toff, ck.cls, m, lane);
+                y0 = ck.e[j].x >> 16;
+                const bool row = (m.w >> 16) != 0x4410;
+                const int c = m.w & 0xFFFF, before = c ? c - 1 : H - 1;
+#pragma unroll
+                for (int u = 0; u < NU; ++u) {
+                    if (touched & (1u << u)) {
+                        const int cur = ck.cur[u][lane];
+                        if (cur >= 0) ck.cur[u][lane] = cur + m.z;
+                    }
+                    // a row move also brings the class row before the one that wraps next to the row past the
+                    // footprint, or away from it
+                    if (row && (ck.cls[u][lane] >> 16) == before) touched |= 1u << u;
+                }
+            }
+        }
+        entry(table + (size_t)zn * PB);
     }
-    if (nbuf) drain(nbuf);
-    return j;
 }
 
-// An entry's placement is consistent with the table and the grid (the checks of the gridder's
-// staging; never false for a work list written by vis_compress for this table and grid).
-__device__ __forceinline__ bool entry_ok(const int4& E, const int* __restrict__ supports, int N, int K, int C,
-                                         int64_t n_samples)
-{
-    const int k = E.w & 0xFFF, ch = (E.w >> 16) & 0xFFFF;
-    if (E.w < 0 || k >= K || ch >= C) return false;
-    const int S = __ldg(&supports[k]);
-    const int x0 = E.x & 0xFFFF, y0 = (E.x >> 16) & 0xFFFF;
-    const int cu = E.y & 0xFFFF, cv = (E.y >> 16) & 0xFFFF;
-    return x0 + S <= N && y0 + S <= N && cu < S && cv < S && E.z >= 0 &&
-           (int64_t)E.z + (int64_t)S * S <= n_samples;
-}
+template <int P>
+constexpr size_t kDegridSmem = Chunk<P, false>::kBytes + kRedFloats * sizeof(float);     // per warp
 
 }  // namespace
 
@@ -294,67 +271,50 @@ __global__ void k_degrid_zero(float4* __restrict__ acc, const long long* __restr
     if (i0 == 0 && (n2 & 1)) reinterpret_cast<float2*>(acc)[n2 - 1] = make_float2(0.f, 0.f);
 }
 
-template <int P, int RT>
-__global__ void __launch_bounds__(kWarps * 32, P == 1 ? 5 : 4) k_degrid_sum(const int4* __restrict__ entries,
-                                                               const int* __restrict__ seg_off,
-                                                               const long long* __restrict__ scal,
-                                                               const int* __restrict__ supports,
-                                                               const float2* __restrict__ table,
-                                                               const float2* __restrict__ grid, int N, int K, int C,
-                                                               int64_t n_samples, int seg_len, int slots,
-                                                               unsigned int* __restrict__ counter,
-                                                               float* __restrict__ acc, long long* __restrict__ dropped)
+template <int P>
+__global__ void __launch_bounds__(kWarps * 32, P == 4 ? 4 : 5) k_degrid_sum(TaskParams tp, const char* __restrict__ table,
+                                                                                        const float2* __restrict__ grid,
+                                                                                        float* __restrict__ acc)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    WarpSmem sm(smem_raw + (size_t)wid * WarpSmem::bytes(seg_len));
-    const long long n_entries = scal[0], n_tasks = scal[1], n_seg = scal[2];
-    const size_t chan_stride = (size_t)N * N * P;
+    unsigned char* base = smem_raw + (size_t)wid * kDegridSmem<P>;
+    Chunk<P, false> ck(base, lane);
+    float* red = reinterpret_cast<float*>(base + Chunk<P, false>::kBytes);
+    const int parts = item_parts(tp);
 
-    for (;;) {
-        unsigned int t = 0;
-        if (lane == 0) t = atomicAdd(counter, 1u);
-        t = __shfl_sync(0xffffffffu, t, 0);
-        if ((long long)t >= n_tasks) break;
-        int lo = 0, hi = (int)n_seg;
-        while (hi - lo > 1) {
-            const int mid = (lo + hi) >> 1;
-            if (__ldg(&seg_off[mid]) <= (int)t) lo = mid; else hi = mid;
-        }
-        const int blk = (int)t - __ldg(&seg_off[lo]);
-        const int e0 = lo * seg_len;
-        const int n = (int)min((long long)seg_len, n_entries - e0);
-
-        __syncwarp();
-        for (int i = lane; i < n; i += 32) cp_async16(&sm.rec[i], entries + e0 + i);
-        asm volatile("cp.async.commit_group;\n" ::);
-        asm volatile("cp.async.wait_group 0;\n" ::);
-        __syncwarp();
-        for (int i = lane; i < n; i += 32) {
-            const int4 E = sm.rec[i];
-            const bool ok = entry_ok(E, supports, N, K, C, n_samples);
-            sm.rec[i].w = ok ? (__ldg(&supports[E.w & 0xFFF]) << 16) | ((E.w >> 16) & 0xFFFF) : -1;
-            if (!ok && blk == 0) atomicAdd(reinterpret_cast<unsigned long long*>(dropped), 1ull);
-        }
-        __syncwarp();
-
-        int j = 0;
-        while (j < n) {
-            const int key = sm.rec[j].w;
-            if (key < 0) {
-                ++j;
-                continue;
+    Item it;
+    while (next_item(tp, parts, lane, it)) {
+        // passes over the entries as in the gridder
+        bool again = it.n > 0;
+        for (int pass = 0; again; ++pass) {
+            again = false;
+            const bool report = it.blk == 0 && pass == 0;
+            ck.begin(tp, it.e0, it.n);
+            int j = 0;
+            while (j >= 0) {
+                if (j == ck.cnt) {
+                    if (!ck.next(tp, report)) break;
+                    j = 0;
+                }
+                const int key = ck.e[j].w;
+                const int S = key_support(key), ch = key_chan(key);
+                const int nb = key < 0 ? 0 : (S * S + tp.slots - 1) / tp.slots;
+                int2 un = make_int2(0, 0);
+                if (it.blk < nb) {       // not a rejected entry, nor a support with fewer blocks
+                    un = block_units(S, it.blk, nb);
+                    if (un.y - un.x > (pass + 1) * kUnitsMax) again = true;
+                    un = make_int2(un.x + pass * kUnitsMax, min(un.y, un.x + (pass + 1) * kUnitsMax));
+                }
+                if (un.x >= un.y) {
+                    j = ck.run_end(j);
+                    continue;
+                }
+                if (P == 4 || un.y - un.x > 2)
+                    j = degrid_entries<P, kUnitsMax>(ck, j, S, ch, un, tp, report, red, table, grid, acc);
+                else
+                    j = degrid_entries<P, 2>(ck, j, S, ch, un, tp, report, red, table, grid, acc);
             }
-            const int S = key >> 16, ch = key & 0xFFFF;
-            const int s2 = S * S;
-            const int nb = (s2 + slots - 1) / slots;
-            const int R = RT > 0 ? RT : (s2 + 32 * nb - 1) / (32 * nb);
-            if (blk >= nb) {     // this block has no points for this support: skip the run
-                while (j < n && sm.rec[j].w == key) ++j;
-                continue;
-            }
-            j = degrid_records<P, RT>(j, n, key, S, R, blk, N, lane, sm, table, grid + (size_t)ch * chan_stride,
-                                      acc + (size_t)e0 * 2 * P);
         }
     }
 }
@@ -436,23 +396,20 @@ __global__ void __launch_bounds__(512) k_degrid_tile(const int2* __restrict__ ru
     }
 }
 
-template <int P, int RT>
+template <int P>
 static int degrid_sum_launch(const Grid& g, const Table& t, const WorkList& wl, cudaStream_t s)
 {
-    static int blocks_per_sm[kSegLenMax / kSegLenMin + 1] = {0};
-    const int smem = (int)(kWarps * WarpSmem::bytes(wl.seg_len));
-    int& bps = blocks_per_sm[wl.seg_len / kSegLenMin];
-    if (bps == 0) {
-        WG_CUDA(cudaFuncSetAttribute(k_degrid_sum<P, RT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)(kWarps * WarpSmem::bytes(kSegLenMax))));
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, k_degrid_sum<P, RT>, kWarps * 32, smem) !=
-                cudaSuccess ||
-            bps < 1)
-            bps = 1;
+    static int blocks_per_sm = 0;
+    const int smem = (int)(kWarps * kDegridSmem<P>);
+    if (blocks_per_sm == 0) {
+        WG_CUDA(cudaFuncSetAttribute(k_degrid_sum<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks_per_sm, k_degrid_sum<P>, kWarps * 32, smem) != cudaSuccess ||
+            blocks_per_sm < 1)
+            blocks_per_sm = 1;
     }
-    k_degrid_sum<P, RT><<<num_sms() * bps, kWarps * 32, smem, s>>>(
-        wl.entries, wl.seg_off, wl.scal, t.supports_d, t.data, g.data, g.n, t.K, g.n_chan, t.n_samples, wl.seg_len,
-        wl.slots, wl.task_counter + 1, reinterpret_cast<float*>(wl.dacc), wl.scal + 3);
+    k_degrid_sum<P><<<num_sms() * blocks_per_sm, kWarps * 32, smem, s>>>(
+        task_params(g, t, wl, wl.task_counter + 1), reinterpret_cast<const char*>(t.pairs), g.data,
+        reinterpret_cast<float*>(wl.dacc));
     WG_LAUNCHED("k_degrid_sum");
     return WG_OK;
 }
@@ -466,10 +423,7 @@ static int degrid_impl(const Grid& g, const Table& t, const wg_vis_in& in, const
     const int zb = num_sms() * 4;
     k_degrid_zero<<<zb, 256, 0, s>>>(reinterpret_cast<float4*>(wl.dacc), wl.scal, P);
     WG_LAUNCHED("k_degrid_zero");
-    int rc;
-    if (wl.fixed_r && wl.slots == 256) rc = degrid_sum_launch<P, 8>(g, t, wl, s);
-    else if (wl.fixed_r && wl.slots == 128) rc = degrid_sum_launch<P, 4>(g, t, wl, s);
-    else rc = degrid_sum_launch<P, 0>(g, t, wl, s);
+    const int rc = degrid_sum_launch<P>(g, t, wl, s);
     if (rc != WG_OK) return rc;
     const int tile_smem = (int)(sizeof(float2) * (size_t)wl.rpb * in.n_chan * P);
     static bool attr_set[5] = {false, false, false, false, false};

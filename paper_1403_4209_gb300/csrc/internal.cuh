@@ -42,13 +42,12 @@ constexpr int kSegLenMin = 32;        // gridded entries per gridder segment: ra
 constexpr int kSegLenMax = 256;
 constexpr int kSegLenDefault = 128;
 constexpr int kSlotsMin = 64;         // footprint points per gridder task: range and default
-constexpr int kSlotsMax = 256;        // (32 lanes x kRMax)
+constexpr int kSlotsMax = 256;
 constexpr int kSlotsDefault = 256;
 static_assert(kSegLenMin == WG_PLAN_SEG_LEN_MIN && kSegLenMax == WG_PLAN_SEG_LEN_MAX &&
                   kSegLenDefault == WG_PLAN_SEG_LEN_DEFAULT && kSlotsMin == WG_PLAN_SLOTS_MIN &&
                   kSlotsMax == WG_PLAN_SLOTS_MAX && kSlotsDefault == WG_PLAN_SLOTS_DEFAULT,
               "plan limits differ from the header's");
-constexpr int kRMax = 8;              // points per lane
 constexpr int kNormSlots = 256;       // privatised normaliser accumulators
 
 // ---- handles --------------------------------------------------------------------------
@@ -106,7 +105,7 @@ struct WorkList {
     int64_t seg_cap = 0;
     int seg_len = kSegLenDefault;         // gridder plan: entries per segment
     int slots = kSlotsDefault;            // gridder plan: footprint points per task
-    bool fixed_r = false;                 // gridder plan: R = slots / 32 for every support
+    bool fixed_r = false;                 // gridder plan: WG_PLAN_FIXED_R (kept, without effect)
     bool interleave = false;              // last batch: channels interleaved onto one grid
     bool cross_swap = false;              // last batch: take-conjugate records swap cross hands
     int wstack_k = 1;                     // last batch: w-stacking planes (1: no stacking)

@@ -5,7 +5,8 @@ than a warp's 32 entries.  Random kernel tables (no symmetry), so that a transpo
 mirrored sample shows.  Reference: the FP64 oracle on the same table and coordinates, held to
 the parity tests' FP32 bar (1e-5 of the norm: sums of a few hundred FP32 products, 6e-8 each).
 
-An infinite or NaN visibility reaches the pixels of its own footprint and no others."""
+An infinite or NaN visibility reaches the pixels of its own footprint and no others; an infinite or
+NaN pixel reaches the visibilities whose footprints hold it and no others."""
 import numpy as np
 import pytest
 import torch
@@ -128,6 +129,43 @@ def test_nonfinite_visibilities_stay_in_their_footprints(P, comp):
     pl0 = oracle.place(batch.uvw.cpu().numpy(), batch.freq.cpu().numpy(), 1.0, N, ref, flag=fl)
     want = oracle.grid_plain(pl0, ref, vis, wt, fl, N)[0, ..., 0]
     assert np.abs(g[..., 0][~hit] - want[~hit]).max() < 1e-5 * np.abs(want).max()
+
+
+@pytest.mark.parametrize("P", [1, 2, 4])
+@pytest.mark.parametrize("supports", SUPPORTS, ids=str)
+def test_degridding_of_edges_walks_and_jumps(supports, P):
+    N, C = 2 * (max(supports) + 20), 2
+    ref, tab, pl, batch, vis, wt, fl = _case(supports, P, N, 700, 9 * P + len(supports), C=C)
+    rng = np.random.default_rng(P)
+    y = (rng.normal(size=(C, N, N, P)) + 1j * rng.normal(size=(C, N, N, P))).astype(np.complex64)
+    want = oracle.degrid(pl, ref, y.astype(np.complex128), wt, fl)
+    for plan in (None, (32, 64, False), (256, 256, True)):
+        g, work = _grid(tab, batch, P, N, C, plan)
+        g.data.copy_(torch.as_tensor(y))
+        got = wg.degrid_vis(g, tab, batch, work).cpu().numpy().reshape(-1, P)
+        assert max_rel(got, want) < 1e-5
+
+
+@pytest.mark.parametrize("P", [1, 4])
+def test_nonfinite_pixels_stay_in_their_footprints(P):
+    # one bad row of pixels: the records whose footprint touches it are not finite, the others are exact
+    # (a footprint that ends on the row above it has that row in its pairs, with zero samples)
+    supports, N = [9, 11], 96
+    ref, tab, pl, batch, vis, wt, fl = _case(supports, P, N, 900, 31)
+    rng = np.random.default_rng(5)
+    y = (rng.normal(size=(1, N, N, P)) + 1j * rng.normal(size=(1, N, N, P))).astype(np.complex64)
+    clean = oracle.degrid(pl, ref, y.astype(np.complex128), wt, fl)
+    row = 50
+    bad = y.copy()
+    bad[0, row] = np.nan
+    bad[0, row, ::2] = np.inf
+    g, work = _grid(tab, batch, P, N, 1, None)
+    g.data.copy_(torch.as_tensor(bad))
+    got = wg.degrid_vis(g, tab, batch, work).cpu().numpy().reshape(-1, P)
+    hit = pl.griddable & (pl.y0 <= row) & (pl.y0 + pl.S > row)
+    assert hit.any() and (pl.griddable & (pl.y0 + pl.S == row)).any()
+    assert not np.isfinite(got[hit]).any() and np.isfinite(got[~hit]).all()
+    assert np.abs(got[~hit] - clean[~hit]).max() < 1e-5 * np.abs(clean).max()
 
 
 def test_degridding_again_with_an_odd_number_of_entries():
