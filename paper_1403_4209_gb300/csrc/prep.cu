@@ -632,11 +632,11 @@ __device__ __forceinline__ unsigned flags_of(const uint8_t* __restrict__ flag, i
 // rank among the tile's gridded records of its list, its entry,
 // gamma and run (first and last row, or record when interleaved); for the compressed records a
 // tile starts with (a carry: the end of a run begun in an earlier tile), their sum in
-// carry[tile][sequence] for k_carry.  Adds zeta(sub-kernel) x sum eps (1-f) to the normaliser.
+// carry[tile][sequence] for k_carry.  wsum becomes the run's normaliser terms, zeta(sub-kernel) x sum eps (1-f).
 template <int P>
 __device__ __forceinline__ void emit_run(const int4& info, bool is_carry, int rank, int64_t tile, int C, int ch,
-                                         int gch, int64_t first, int64_t last, const float2 (&acc)[P], const float (&wsum)[P],
-                                         const PlaceParams& pp, float* s_norm, const int* __restrict__ tile_off,
+                                         int gch, int64_t first, int64_t last, const float2 (&acc)[P], float (&wsum)[P],
+                                         const PlaceParams& pp, const int* __restrict__ tile_off,
                                          const int* __restrict__ chan_base, int4* __restrict__ entries,
                                          float2* __restrict__ gamma, int2* __restrict__ runs, int64_t cap_entries,
                                          float2* __restrict__ carry_q, int* __restrict__ carry_last,
@@ -647,8 +647,7 @@ __device__ __forceinline__ void emit_run(const int4& info, bool is_carry, int ra
     const int sub = (info.z - __ldg(&pp.offsets[k])) / (S * S);
     const float zeta = __ldg(&pp.zeta_f[k * pp.beta * pp.beta + sub]);
 #pragma unroll
-    for (int p = 0; p < P; ++p)
-        if (wsum[p] != 0.f) atomicAdd(&s_norm[gch * P + p], zeta * wsum[p]);
+    for (int p = 0; p < P; ++p) wsum[p] = zeta * wsum[p];
     if (is_carry) {
         const int64_t c = tile * C + gch;
 #pragma unroll
@@ -667,8 +666,14 @@ __device__ __forceinline__ void emit_run(const int4& info, bool is_carry, int ra
     const int rx = mod_small(info.x & 0xFFFF, S, inv_s), ry = mod_small((info.x >> 16) & 0xFFFF, S, inv_s);
     const int cuv = (rx ? S - rx : 0) | ((ry ? S - ry : 0) << 16);
     entries[dst] = make_int4(info.x, cuv, info.z, k | (ech << 16));
+    if constexpr (P == 1) {
+        gamma[dst] = acc[0];
+    } else {
 #pragma unroll
-    for (int p = 0; p < P; ++p) gamma[(int64_t)dst * P + p] = acc[p];
+        for (int h = 0; h < P; h += 2)
+            *reinterpret_cast<float4*>(gamma + (int64_t)dst * P + h) =
+                make_float4(acc[h].x, acc[h].y, acc[h + 1].x, acc[h + 1].y);
+    }
     runs[dst] = make_int2((int)first, (int)last);
 }
 
@@ -703,8 +708,7 @@ __global__ void __launch_bounds__(kCompactThreads, 2) k_compact(const int4* __re
     const int cap = rpb * C;
     float2* s_q = reinterpret_cast<float2*>(smem);                        // [P][cap] or [cap][P]
     float* s_w = reinterpret_cast<float*>(s_q + (size_t)cap * P);         // [P][cap] or [cap][P]
-    float* s_norm = s_w + (size_t)cap * P;                                // [C][P]
-    int* s_heads = reinterpret_cast<int*>(s_norm + (size_t)C * P);        // [cap]
+    int* s_heads = reinterpret_cast<int*>(s_w + (size_t)cap * P);         // [cap]
     uint8_t* s_cls = reinterpret_cast<uint8_t*>(s_heads + cap);           // [cap]
     int* s_first = reinterpret_cast<int*>(s_cls + ((cap + 3) & ~3));     // [C]: list position of each channel's first head
     __shared__ int s_wtot[kCompactThreads / 32];
@@ -736,7 +740,6 @@ __global__ void __launch_bounds__(kCompactThreads, 2) k_compact(const int4* __re
         }
     }
     if (threadIdx.x == 0) s_abort = 0;
-    for (int i = threadIdx.x; i < C * P; i += blockDim.x) s_norm[i] = 0.f;
     __syncthreads();
     if constexpr (BULK) {
         constexpr int kU = 4;                    // records per thread whose class and flag loads are issued together
@@ -938,13 +941,26 @@ __global__ void __launch_bounds__(kCompactThreads, 2) k_compact(const int4* __re
         }
         const int64_t last = IL ? row0 * C + jl : row0 + jl / C;
         const int rank = is_carry ? 0 : (IL ? h : h - s_first[ch]);
-        emit_run<P>(info, is_carry, rank, tile, C, ch, gch, IL ? rec : row, last, acc, wsum, pp, s_norm, tile_off,
+        emit_run<P>(info, is_carry, rank, tile, C, ch, gch, IL ? rec : row, last, acc, wsum, pp, tile_off,
                     chan_base, entries, gamma, runs, cap_entries, carry_q, carry_last, scal);
+        // the run's normaliser terms take the place of its first record's weights (no other run reads them)
+#pragma unroll
+        for (int p = 0; p < P; ++p) s_w[BULK ? j * P + p : p * cap + j] = wsum[p];
     }
     __syncthreads();
+    // The tile's part of N_p: one thread per channel and polarisation adds the terms of its runs in list order,
+    // in FP32 (as shared-memory atomics, compare-and-swap loops on one address a channel, they took a
+    // third of the kernel's shared-memory wavefronts, and 40 of 59 us where every record starts a run).
     const int slot = (int)(tile % kNormSlots);
-    for (int i = threadIdx.x; i < C * P; i += blockDim.x)
-        if (s_norm[i] != 0.f) atomicAdd(&norm_priv[(int64_t)slot * C * P + i], (double)s_norm[i]);
+    for (int i = threadIdx.x; i < n_seq * P; i += blockDim.x) {
+        const int ch = i / P, p = i - ch * P;
+        const float* w = s_w + (BULK ? p : p * cap);
+        float sum = (s_cls[ch] & 2) ? w[BULK ? ch * P : ch] : 0.f;       // the carry
+        const int h0 = IL ? 0 : s_first[ch], h1 = IL || ch + 1 == C ? nh : s_first[ch + 1];
+#pragma unroll 8
+        for (int h = h0; h < h1; ++h) sum += w[BULK ? s_heads[h] * P : s_heads[h]];
+        if (sum != 0.f) atomicAdd(&norm_priv[(int64_t)slot * C * P + i], (double)sum);
+    }
 }
 
 // adds each tile's carried run part (compressed records continuing a run of an earlier tile) to
