@@ -104,13 +104,14 @@ int grid_create(const wg_grid_desc* d, wg_grid** out)
         g.owns = true;
     }
     g.comp = (d->flags & WG_GRID_COMPENSATED) != 0;
-    if (dev_malloc((void**)&g.norm, sizeof(double) * g.n_chan * g.n_pol) != cudaSuccess ||
-        dev_malloc((void**)&g.counters, sizeof(unsigned long long) * ST_N) != cudaSuccess ||
+    // the counters follow the normaliser in one buffer, so that grid_zero clears both at once
+    if (dev_malloc((void**)&g.norm, sizeof(double) * g.n_chan * g.n_pol + sizeof(unsigned long long) * ST_N) != cudaSuccess ||
         (g.comp && dev_malloc((void**)&g.err, bytes) != cudaSuccess)) {
         cudaGetLastError();
         grid_destroy(h);
         return fail(WG_E_OOM, "cannot allocate normaliser");
     }
+    g.counters = reinterpret_cast<unsigned long long*>(g.norm + (size_t)g.n_chan * g.n_pol);
     int rc = grid_zero(h, nullptr);
     if (rc == WG_OK && cudaDeviceSynchronize() != cudaSuccess) rc = cuda_fail(cudaGetLastError(), "grid_create");
     if (rc != WG_OK) {
@@ -127,7 +128,6 @@ int grid_destroy(wg_grid* h)
     Grid& g = h->g;
     if (g.owns) cudaFree(g.data);
     cudaFree(g.norm);
-    cudaFree(g.counters);
     cudaFree(g.err);
     cudaFree(g.scratch);
     cudaFree(g.corr);
@@ -145,8 +145,7 @@ int grid_zero(wg_grid* h, void* stream)
     Grid& g = h->g;
     WG_CUDA(cudaMemsetAsync(g.data, 0, sizeof(float2) * (size_t)g.n * g.n * g.n_pol * g.n_chan, S(stream)));
     if (g.err) WG_CUDA(cudaMemsetAsync(g.err, 0, sizeof(float2) * (size_t)g.n * g.n * g.n_pol * g.n_chan, S(stream)));
-    WG_CUDA(cudaMemsetAsync(g.norm, 0, sizeof(double) * g.n_chan * g.n_pol, S(stream)));
-    WG_CUDA(cudaMemsetAsync(g.counters, 0, sizeof(unsigned long long) * ST_N, S(stream)));
+    WG_CUDA(cudaMemsetAsync(g.norm, 0, sizeof(double) * g.n_chan * g.n_pol + sizeof(unsigned long long) * ST_N, S(stream)));
     return WG_OK;
 }
 

@@ -262,9 +262,10 @@ constexpr size_t kDegridSmem = Chunk<P, false>::kBytes + kRedFloats * sizeof(flo
 
 }  // namespace
 
-// acc[0 .. n_entries * 2P) = 0
-__global__ void k_degrid_zero(float4* __restrict__ acc, const long long* __restrict__ scal, int P)
+// acc[0 .. n_entries * 2P) = 0, and k_degrid_sum's task counter
+__global__ void k_degrid_zero(float4* __restrict__ acc, const long long* __restrict__ scal, int P, unsigned* __restrict__ counter)
 {
+    if (blockIdx.x == 0 && threadIdx.x == 0) *counter = 0u;
     const long long n2 = scal[0] * P, n4 = n2 / 2;
     const long long i0 = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     for (long long i = i0; i < n4; i += (long long)gridDim.x * blockDim.x) acc[i] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -419,9 +420,8 @@ static int degrid_impl(const Grid& g, const Table& t, const wg_vis_in& in, const
                        cudaStream_t s)
 {
     if (!wl.dacc) return fail(WG_E_INVALID_ARG, "degrid_vis: the work list has no degridding accumulator");
-    WG_CUDA(cudaMemsetAsync(wl.task_counter + 1, 0, sizeof(unsigned int), s));
     const int zb = num_sms() * 4;
-    k_degrid_zero<<<zb, 256, 0, s>>>(reinterpret_cast<float4*>(wl.dacc), wl.scal, P);
+    k_degrid_zero<<<zb, 256, 0, s>>>(reinterpret_cast<float4*>(wl.dacc), wl.scal, P, wl.task_counter + 1);
     WG_LAUNCHED("k_degrid_zero");
     const int rc = degrid_sum_launch<P>(g, t, wl, s);
     if (rc != WG_OK) return rc;

@@ -16,7 +16,7 @@
 //               walks its run of compressed successors and sums eps (1-f) psi-conj(vis) (a run
 //               crossing a tile end is finished by k_carry from the next tiles' carries); the
 //               run's eps (1-f) times its sub-kernel's zeta gives the normaliser terms (eq.
-//               "normalizer"), summed by k_norm_sum.
+//               "normalizer"), summed in the same launch as the carries (k_carry).
 //   k_segments + k_seg_scan (Plan Create / Plan Analyse, Algorithm "plan"): gridded entries
 //               are cut into segments of seg_len entries; each segment needs one gridder task
 //               per block of `slots` footprint points of its largest support.  The plan can be
@@ -281,17 +281,38 @@ __device__ __forceinline__ int nblk_of(int S, int slots)
 
 }  // namespace
 
-__global__ void k_chan_scale(const double* __restrict__ freq, int C, double beta_over_du, double* lam_inv,
-                             double* sc, float* lam_f, float* sc_f)
+__device__ __forceinline__ void chan_scale(const double* __restrict__ freq, int c, double beta_over_du, double* lam_inv,
+                                           double* sc, float* lam_f, float* sc_f)
 {
-    int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= C) return;
     const double li = __ddiv_rn(freq[c], 299792458.0);
     const double s = __dmul_rn(li, beta_over_du);
     lam_inv[c] = li;
     sc[c] = s;
     lam_f[c] = __double2float_rn(li);
     sc_f[c] = __double2float_rn(s);
+}
+
+__global__ void k_chan_scale(const double* __restrict__ freq, int C, double beta_over_du, double* lam_inv,
+                             double* sc, float* lam_f, float* sc_f)
+{
+    const int c = blockIdx.x * blockDim.x + threadIdx.x;
+    if (c < C) chan_scale(freq, c, beta_over_du, lam_inv, sc, lam_f, sc_f);
+}
+
+// What a batch starts from, in one launch: the channel scales, and zero in the privatised normaliser and
+// statistics, the statistics and the counts.  An appended batch keeps the entry count and the dropped
+// count of the earlier ones (scal[0], scal[3]) and the summed statistics; its plan is redone.
+__global__ void k_prep_init(const double* __restrict__ freq, int C, double beta_over_du, double* lam_inv, double* sc,
+                            float* lam_f, float* sc_f, double* __restrict__ norm_priv, int64_t n_norm,
+                            unsigned long long* __restrict__ stat_priv, unsigned long long* __restrict__ stats,
+                            long long* __restrict__ scal, int append)
+{
+    const int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, n = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t i = i0; i < n_norm; i += n) norm_priv[i] = 0.0;
+    for (int64_t i = i0; i < kNormSlots * ST_N; i += n) stat_priv[i] = 0ull;
+    for (int64_t i = i0; i < C; i += n) chan_scale(freq, (int)i, beta_over_du, lam_inv, sc, lam_f, sc_f);
+    if (i0 < ST_N && !append) stats[i0] = 0ull;
+    if (i0 < 4 && (!append || i0 == 1 || i0 == 2)) scal[i0] = 0;
 }
 
 template <int P>
@@ -417,71 +438,114 @@ __global__ void __launch_bounds__(512, 3) k_classify(const double* __restrict__ 
         atomicAdd(&stat_priv[slot * ST_N + threadIdx.x], s_stat[threadIdx.x]);
 }
 
-// per-channel exclusive scan of tile counts over tiles
+// Inclusive scan of v over the block (blockDim a multiple of 32); warp_tot: shared scratch of 32 ints.
+// Returns the thread's inclusive prefix; total is the block's sum.
+__device__ __forceinline__ int block_inclusive(int v, int* warp_tot, int& total)
+{
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    for (int o = 1; o < 32; o <<= 1) {
+        const int u = __shfl_up_sync(0xffffffffu, v, o);
+        if (lane >= o) v += u;
+    }
+    if (lane == 31) warp_tot[wid] = v;
+    __syncthreads();
+    if (wid == 0) {
+        int x = lane < nw ? warp_tot[lane] : 0;
+        for (int o = 1; o < 32; o <<= 1) {
+            const int u = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += u;
+        }
+        warp_tot[lane] = x;
+    }
+    __syncthreads();
+    if (wid > 0) v += warp_tot[wid - 1];
+    total = warp_tot[nw - 1];
+    __syncthreads();
+    return v;
+}
+
+// Per-channel exclusive scan of tile counts over tiles (one block a channel).  A thread takes kScan tiles a
+// step, whose loads are under way together: a step's time is one round trip and its barriers,
+// whatever it covers.
+constexpr int kScan = 8;
 __global__ void __launch_bounds__(1024) k_scan_tiles(int* __restrict__ tile_cnt, int64_t n_tiles, int C,
                                                      int* __restrict__ chan_total)
 {
     __shared__ int warp_tot[32];
-    __shared__ int carry_s;
     const int ch = blockIdx.x;
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     int carry = 0;
-    for (int64_t base = 0; base < n_tiles; base += blockDim.x) {
-        const int64_t t = base + threadIdx.x;
-        const int v = (t < n_tiles) ? tile_cnt[t * C + ch] : 0;
-        int inc = v;
-        for (int o = 1; o < 32; o <<= 1) {
-            int u = __shfl_up_sync(0xffffffffu, inc, o);
-            if (lane >= o) inc += u;
+    for (int64_t base = 0; base < n_tiles; base += (int64_t)blockDim.x * kScan) {
+        const int64_t t0 = base + (int64_t)threadIdx.x * kScan;
+        int v[kScan], sum = 0, total;
+#pragma unroll
+        for (int i = 0; i < kScan; ++i) v[i] = (t0 + i < n_tiles) ? tile_cnt[(t0 + i) * C + ch] : 0;
+#pragma unroll
+        for (int i = 0; i < kScan; ++i) sum += v[i];
+        int at = carry + block_inclusive(sum, warp_tot, total) - sum;
+#pragma unroll
+        for (int i = 0; i < kScan; ++i) {
+            if (t0 + i < n_tiles) tile_cnt[(t0 + i) * C + ch] = at;
+            at += v[i];
         }
-        if (lane == 31) warp_tot[wid] = inc;
-        __syncthreads();
-        if (wid == 0) {
-            int x = (lane < (int)(blockDim.x >> 5)) ? warp_tot[lane] : 0;
-            for (int o = 1; o < 32; o <<= 1) {
-                int u = __shfl_up_sync(0xffffffffu, x, o);
-                if (lane >= o) x += u;
-            }
-            warp_tot[lane] = x;
-        }
-        __syncthreads();
-        const int excl = carry + inc - v + (wid > 0 ? warp_tot[wid - 1] : 0);
-        if (t < n_tiles) tile_cnt[t * C + ch] = excl;
-        if (threadIdx.x == blockDim.x - 1) carry_s = carry + warp_tot[(blockDim.x >> 5) - 1];
-        __syncthreads();
-        carry = carry_s;
-        __syncthreads();
+        carry += total;
     }
     if (threadIdx.x == 0) chan_total[ch] = carry;
 }
 
-__global__ void k_finalize(int* __restrict__ chan_base, int C, const unsigned long long* __restrict__ stat_priv,
-                           unsigned long long* __restrict__ stats, unsigned long long* __restrict__ stats_batch,
-                           long long* __restrict__ scal, long long cap, int append)
+// One block of kNormSlots threads: the channel bases, and the sums of the privatised statistics.  The channel
+// totals go through shared memory a chunk at a time and each slot's counters are loaded by a thread of its
+// own (one thread walking global memory took 15 us whatever the batch).
+__global__ void __launch_bounds__(kNormSlots) k_finalize(int* __restrict__ chan_base, int C,
+                                                         const unsigned long long* __restrict__ stat_priv,
+                                                         unsigned long long* __restrict__ stats,
+                                                         unsigned long long* __restrict__ stats_batch,
+                                                         long long* __restrict__ scal, long long cap, int append)
 {
-    if (threadIdx.x == 0) {
-        // channel bases and the entry count, held to the work list's capacity (a count past it
-        // is reported as dropped); an appended batch's entries follow those already listed
-        long long run = append ? scal[0] : 0;
-        bool over = false;
-        for (int c = 0; c < C; ++c) {
-            const int t = chan_base[c];
-            chan_base[c] = (int)run;
-            run += t;
-            if (t < 0 || run > cap) {
-                over = true;
-                run = t < 0 ? run - t : cap;
+    __shared__ int s_tot[kNormSlots];
+    __shared__ unsigned long long s_stat[ST_TASKS];
+    if (threadIdx.x < ST_TASKS) s_stat[threadIdx.x] = 0ull;
+    unsigned long long v[ST_TASKS];
+#pragma unroll
+    for (int q = 0; q < ST_TASKS; ++q) v[q] = stat_priv[threadIdx.x * ST_N + q];
+    // channel bases and the entry count, held to the work list's capacity (a count past it
+    // is reported as dropped); an appended batch's entries follow those already listed
+    long long run = append ? scal[0] : 0;
+    bool over = false;
+    for (int c0 = 0; c0 < C; c0 += kNormSlots) {
+        const int n = min(kNormSlots, C - c0);
+        __syncthreads();
+        if ((int)threadIdx.x < n) s_tot[threadIdx.x] = chan_base[c0 + threadIdx.x];
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            for (int c = 0; c < n; ++c) {
+                const int t = s_tot[c];
+                s_tot[c] = (int)run;
+                run += t;
+                if (t < 0 || run > cap) {
+                    over = true;
+                    run = t < 0 ? run - t : cap;
+                }
             }
         }
+        __syncthreads();
+        if ((int)threadIdx.x < n) chan_base[c0 + threadIdx.x] = s_tot[threadIdx.x];
+    }
+    if (threadIdx.x == 0) {
         chan_base[C] = (int)run;
         scal[0] = run;
         if (over) atomicAdd(reinterpret_cast<unsigned long long*>(&scal[3]), 1ull);
     }
-    for (int q = threadIdx.x; q < ST_TASKS; q += blockDim.x) {
-        unsigned long long s = 0;
-        for (int k = 0; k < kNormSlots; ++k) s += stat_priv[k * ST_N + q];
-        stats_batch[q] = s;
-        stats[q] = append ? stats[q] + s : s;
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < ST_TASKS; ++q) {
+        for (int o = 16; o > 0; o >>= 1) v[q] += __shfl_xor_sync(0xffffffffu, v[q], o);
+        if ((threadIdx.x & 31) == 0 && v[q]) atomicAdd(&s_stat[q], v[q]);
+    }
+    __syncthreads();
+    if (threadIdx.x < ST_TASKS) {
+        const unsigned long long s = s_stat[threadIdx.x];
+        stats_batch[threadIdx.x] = s;
+        stats[threadIdx.x] = append ? stats[threadIdx.x] + s : s;
     }
 }
 
@@ -963,14 +1027,28 @@ __global__ void __launch_bounds__(kCompactThreads, 2) k_compact(const int4* __re
     }
 }
 
-// adds each tile's carried run part (compressed records continuing a run of an earlier tile) to
-// that run's entry, the last entry of the sequence before the tile, and extends the run's end
+// The first carry_blocks blocks add each tile's carried run part (compressed records continuing a run of an
+// earlier tile) to that run's entry, the last entry of the sequence before the tile, and extend the run's
+// end.  The others write N_p of the batch, the sums of the privatised per-slot partials, one warp a sum (one
+// thread a sum took 13 to 23 us in 256 dependent steps).
 template <int P>
 __global__ void k_carry(const float2* __restrict__ carry_q, const int* __restrict__ carry_last, int64_t n_tiles, int C,
                         int n_seq, const int* __restrict__ tile_off, const int* __restrict__ chan_base,
                         float2* __restrict__ gamma, int2* __restrict__ runs, int64_t cap_entries,
-                        long long* __restrict__ scal)
+                        long long* __restrict__ scal, int carry_blocks, const double* __restrict__ norm_priv,
+                        double* __restrict__ norm_batch)
 {
+    if ((int)blockIdx.x >= carry_blocks) {
+        const int lane = threadIdx.x & 31, n = C * P;
+        const int i = (int)(((blockIdx.x - carry_blocks) * blockDim.x + threadIdx.x) >> 5);
+        if (i >= n) return;
+        double s = 0.0;
+#pragma unroll
+        for (int k = 0; k < kNormSlots / 32; ++k) s += norm_priv[(int64_t)(k * 32 + lane) * n + i];
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (lane == 0) norm_batch[i] = s;
+        return;
+    }
     const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;   // tile * C + sequence
     if (c >= n_tiles * C) return;
     const int seq = (int)(c % C);
@@ -991,73 +1069,49 @@ __global__ void k_carry(const float2* __restrict__ carry_q, const int* __restric
     atomicMax(reinterpret_cast<int*>(&runs[dst]) + 1, last);
 }
 
-// N_p of the batch: the sum of the privatised per-slot partials
-__global__ void k_norm_sum(const double* __restrict__ norm_priv, int n, double* __restrict__ norm_batch)
-{
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-        double s = 0.0;
-        for (int k = 0; k < kNormSlots; ++k) s += norm_priv[(int64_t)k * n + i];
-        norm_batch[i] = s;
-    }
-}
-
-// per segment, the number of task blocks of its largest support; sets the segment count
+// per segment, the number of task blocks of its largest support (one warp a segment); sets the segment count
 __global__ void k_segments(const int4* __restrict__ entries, long long* __restrict__ scal,
                            const int* __restrict__ supports, int K, int seg_len, int slots,
                            int* __restrict__ seg_nblk)
 {
-    const long long n = scal[0];
-    if (blockIdx.x == 0 && threadIdx.x == 0) scal[2] = (n + seg_len - 1) / seg_len;
-    // seg_len is a multiple of 32, so the 32 entries of a warp's chunk share one segment: the
-    // warp takes their maximum and one lane updates the segment
+    const long long n = scal[0], n_seg = (n + seg_len - 1) / seg_len;
+    if (blockIdx.x == 0 && threadIdx.x == 0) scal[2] = n_seg;
     const int lane = threadIdx.x & 31;
-    const long long warp0 = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const long long n_warps = ((long long)gridDim.x * blockDim.x) >> 5;
-    for (long long base = warp0 * 32; base < n; base += n_warps * 32) {
-        const long long e = base + lane;
+    for (long long g = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; g < n_seg; g += n_warps) {
+        const int len = (int)min((long long)seg_len, n - g * seg_len);
+        const int4* e = entries + g * seg_len;
         int nb = 0;
-        if (e < n) {
-            const int k = entries[e].w & 0xFFF;
-            nb = (k < K) ? nblk_of(__ldg(&supports[k]), slots) : 1;
+        for (int i = lane; i < len; i += 32) {
+            const int k = e[i].w & 0xFFF;
+            nb = max(nb, (k < K) ? nblk_of(__ldg(&supports[k]), slots) : 1);
         }
-        const int m = __reduce_max_sync(0xffffffffu, nb);
-        if (lane == 0) atomicMax(&seg_nblk[base / seg_len], m);
+        nb = __reduce_max_sync(0xffffffffu, nb);
+        if (lane == 0) seg_nblk[g] = nb;
     }
 }
 
+// exclusive scan of the segments' task counts (one block; kScan segments a thread and step, as above)
 __global__ void __launch_bounds__(1024) k_seg_scan(const int* __restrict__ seg_nblk, int* __restrict__ seg_off,
                                                    long long* __restrict__ scal, unsigned long long* __restrict__ stats)
 {
     __shared__ int warp_tot[32];
-    __shared__ int carry_s;
     const long long n_seg = scal[2];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     int carry = 0;
-    for (long long base = 0; base < n_seg; base += blockDim.x) {
-        const long long t = base + threadIdx.x;
-        const int v = (t < n_seg) ? seg_nblk[t] : 0;
-        int inc = v;
-        for (int o = 1; o < 32; o <<= 1) {
-            int u = __shfl_up_sync(0xffffffffu, inc, o);
-            if (lane >= o) inc += u;
+    for (long long base = 0; base < n_seg; base += (long long)blockDim.x * kScan) {
+        const long long t0 = base + (long long)threadIdx.x * kScan;
+        int v[kScan], sum = 0, total;
+#pragma unroll
+        for (int i = 0; i < kScan; ++i) v[i] = (t0 + i < n_seg) ? seg_nblk[t0 + i] : 0;
+#pragma unroll
+        for (int i = 0; i < kScan; ++i) sum += v[i];
+        int at = carry + block_inclusive(sum, warp_tot, total) - sum;
+#pragma unroll
+        for (int i = 0; i < kScan; ++i) {
+            if (t0 + i < n_seg) seg_off[t0 + i] = at;
+            at += v[i];
         }
-        if (lane == 31) warp_tot[wid] = inc;
-        __syncthreads();
-        if (wid == 0) {
-            int x = (lane < (int)(blockDim.x >> 5)) ? warp_tot[lane] : 0;
-            for (int o = 1; o < 32; o <<= 1) {
-                int u = __shfl_up_sync(0xffffffffu, x, o);
-                if (lane >= o) x += u;
-            }
-            warp_tot[lane] = x;
-        }
-        __syncthreads();
-        const int excl = carry + inc - v + (wid > 0 ? warp_tot[wid - 1] : 0);
-        if (t < n_seg) seg_off[t] = excl;
-        if (threadIdx.x == blockDim.x - 1) carry_s = carry + warp_tot[(blockDim.x >> 5) - 1];
-        __syncthreads();
-        carry = carry_s;
-        __syncthreads();
+        carry += total;
     }
     if (threadIdx.x == 0) {
         seg_off[n_seg] = carry;
@@ -1072,6 +1126,7 @@ static size_t classify_smem(int rpb, int C)
     return cap * sizeof(int4) + (cap + 1) * sizeof(int) + (rpb + 1) * 16 + cap + 16;
 }
 
+// (C P floats of it are not used: they keep the number of channels that are accepted)
 static size_t compact_smem(int rpb, int C, int P)
 {
     const size_t cap = (size_t)rpb * C;
@@ -1143,18 +1198,11 @@ static int prep_impl(const Table& t, const Grid& g, const wg_vis_in& in, int fla
     float* lam_f = reinterpret_cast<float*>(sc + C);                              // [C]
     float* sc_f = lam_f + C;                                                      // [C]
 
-    WG_CUDA(cudaMemsetAsync(wl.norm_priv, 0, sizeof(double) * kNormSlots * C * P, s));
-    WG_CUDA(cudaMemsetAsync(wl.stat_priv, 0, sizeof(unsigned long long) * kNormSlots * ST_N, s));
-    if (app) {
-        // keep the entry count and the dropped count of the earlier batches; the plan is redone
-        WG_CUDA(cudaMemsetAsync(wl.scal + 1, 0, sizeof(long long) * 2, s));
-    } else {
-        WG_CUDA(cudaMemsetAsync(wl.stats, 0, sizeof(unsigned long long) * ST_N, s));
-        WG_CUDA(cudaMemsetAsync(wl.scal, 0, sizeof(long long) * 4, s));
-    }
-
-    k_chan_scale<<<(C + 127) / 128, 128, 0, s>>>(in.freq_hz, C, pp.beta_over_du, lam_inv, sc, lam_f, sc_f);
-    WG_LAUNCHED("k_chan_scale");
+    const int64_t n_norm = (int64_t)kNormSlots * C * P;
+    k_prep_init<<<(unsigned)std::min<int64_t>((std::max<int64_t>(n_norm, C) + 255) / 256, num_sms()), 256, 0, s>>>(
+        in.freq_hz, rows > 0 ? C : 0, pp.beta_over_du, lam_inv, sc, lam_f, sc_f, wl.norm_priv, n_norm, wl.stat_priv, wl.stats,
+        wl.scal, app ? 1 : 0);
+    WG_LAUNCHED("k_prep_init");
     if (rows > 0) {
         const size_t sm = classify_smem(rpb, C);
         if (sm > 48 * 1024) WG_CUDA(cudaFuncSetAttribute(k_classify<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
@@ -1164,7 +1212,7 @@ static int prep_impl(const Table& t, const Grid& g, const wg_vis_in& in, int fla
     }
     k_scan_tiles<<<C, 1024, 0, s>>>(wl.tile_cnt, n_tiles, C, wl.chan_base);
     WG_LAUNCHED("k_scan_tiles");
-    k_finalize<<<1, 256, 0, s>>>(wl.chan_base, C, wl.stat_priv, wl.stats, wl.stats_batch, wl.scal, wl.ecap, app ? 1 : 0);
+    k_finalize<<<1, kNormSlots, 0, s>>>(wl.chan_base, C, wl.stat_priv, wl.stats, wl.stats_batch, wl.scal, wl.ecap, app ? 1 : 0);
     WG_LAUNCHED("k_finalize");
     if (rows > 0) {
         const size_t sm = compact_smem(rpb, C, P);
@@ -1205,15 +1253,13 @@ static int prep_impl(const Table& t, const Grid& g, const wg_vis_in& in, int fla
         if (rc != WG_OK) return rc;
         WG_LAUNCHED("k_compact");
     }
-    if (rows > 0) {
-        const int64_t nc = n_tiles * C;
-        k_carry<P><<<(unsigned)((nc + 255) / 256), 256, 0, s>>>(wl.carry_q, wl.carry_last, n_tiles, C,
-                                                                 pp.interleave ? 1 : C, wl.tile_cnt, wl.chan_base,
-                                                                 wl.gamma, wl.runs, wl.ecap, wl.scal);
+    {
+        const int64_t carry_blocks = (n_tiles * C + 255) / 256;
+        k_carry<P><<<(unsigned)(carry_blocks + (C * P + 7) / 8), 256, 0, s>>>(
+            wl.carry_q, wl.carry_last, n_tiles, C, pp.interleave ? 1 : C, wl.tile_cnt, wl.chan_base, wl.gamma, wl.runs,
+            wl.ecap, wl.scal, (int)carry_blocks, wl.norm_priv, wl.norm_batch);
         WG_LAUNCHED("k_carry");
     }
-    k_norm_sum<<<1, 256, 0, s>>>(wl.norm_priv, C * P, wl.norm_batch);
-    WG_LAUNCHED("k_norm_sum");
     if (app) {
         // the batch's N_p terms and statistics go into its grid channels now; the plan over
         // every appended batch is made by the next grid_vis (or worklist_plan)
@@ -1226,9 +1272,7 @@ static int prep_impl(const Table& t, const Grid& g, const wg_vis_in& in, int fla
 
 int launch_plan(const Table& t, WorkList& wl, cudaStream_t s)
 {
-    const int64_t n_seg_max = (wl.ecap + wl.seg_len - 1) / wl.seg_len + 1;
-    WG_CUDA(cudaMemsetAsync(wl.seg_nblk, 0, sizeof(int) * std::min<int64_t>(n_seg_max, wl.seg_cap), s));
-    k_segments<<<num_sms() * 4, 256, 0, s>>>(wl.entries, wl.scal, t.supports_d, t.K, wl.seg_len, wl.slots,
+    k_segments<<<num_sms() * 8, 256, 0, s>>>(wl.entries, wl.scal, t.supports_d, t.K, wl.seg_len, wl.slots,
                                               wl.seg_nblk);
     WG_LAUNCHED("k_segments");
     k_seg_scan<<<1, 1024, 0, s>>>(wl.seg_nblk, wl.seg_off, wl.scal, wl.stats);
