@@ -778,6 +778,7 @@ __global__ void __launch_bounds__(kCompactThreads, 2) k_compact(const int4* __re
     __shared__ int s_wtot[kCompactThreads / 32];
     __shared__ int s_abort;
     __shared__ unsigned long long s_bar;
+    __shared__ float s_norm[P];                  // interleaved: the tile's normaliser terms
     const int unweighted = pp.unweighted;
 
     // the bulk copies cover whole 16-byte units of the tile's visibilities and weights; a
@@ -804,6 +805,7 @@ __global__ void __launch_bounds__(kCompactThreads, 2) k_compact(const int4* __re
         }
     }
     if (threadIdx.x == 0) s_abort = 0;
+    if (threadIdx.x < P) s_norm[threadIdx.x] = 0.f;
     __syncthreads();
     if constexpr (BULK) {
         constexpr int kU = 4;                    // records per thread whose class and flag loads are issued together
@@ -1007,22 +1009,35 @@ __global__ void __launch_bounds__(kCompactThreads, 2) k_compact(const int4* __re
         const int rank = is_carry ? 0 : (IL ? h : h - s_first[ch]);
         emit_run<P>(info, is_carry, rank, tile, C, ch, gch, IL ? rec : row, last, acc, wsum, pp, tile_off,
                     chan_base, entries, gamma, runs, cap_entries, carry_q, carry_last, scal);
-        // the run's normaliser terms take the place of its first record's weights (no other run reads them)
+        // The run's normaliser terms take the place of its first record's weights (no other run reads them).
+        // Interleaved, the whole tile is one list: its terms are added as they come (an FP32 sum of 2048
+        // terms in list order lies 1e-8 of N_p off that, several times what it varies by).
 #pragma unroll
-        for (int p = 0; p < P; ++p) s_w[BULK ? j * P + p : p * cap + j] = wsum[p];
+        for (int p = 0; p < P; ++p) {
+            if constexpr (IL) {
+                if (wsum[p] != 0.f) atomicAdd(&s_norm[p], wsum[p]);
+            } else {
+                s_w[BULK ? j * P + p : p * cap + j] = wsum[p];
+            }
+        }
     }
     __syncthreads();
     // The tile's part of N_p: one thread per channel and polarisation adds the terms of its runs in list order,
     // in FP32 (as shared-memory atomics, compare-and-swap loops on one address a channel, they took a
-    // third of the kernel's shared-memory wavefronts, and 40 of 59 us where every record starts a run).
+    // third of the kernel's shared-memory wavefronts, and 32 of 59 us where every record starts a run).
     const int slot = (int)(tile % kNormSlots);
     for (int i = threadIdx.x; i < n_seq * P; i += blockDim.x) {
-        const int ch = i / P, p = i - ch * P;
-        const float* w = s_w + (BULK ? p : p * cap);
-        float sum = (s_cls[ch] & 2) ? w[BULK ? ch * P : ch] : 0.f;       // the carry
-        const int h0 = IL ? 0 : s_first[ch], h1 = IL || ch + 1 == C ? nh : s_first[ch + 1];
+        float sum = 0.f;
+        if constexpr (IL) {
+            sum = s_norm[i];
+        } else {
+            const int ch = i / P, p = i - ch * P;
+            const float* w = s_w + (BULK ? p : p * cap);
+            const int h0 = s_first[ch], h1 = ch + 1 == C ? nh : s_first[ch + 1];
 #pragma unroll 8
-        for (int h = h0; h < h1; ++h) sum += w[BULK ? s_heads[h] * P : s_heads[h]];
+            for (int h = h0; h < h1; ++h) sum += w[BULK ? s_heads[h] * P : s_heads[h]];
+            if (s_cls[ch] & 2) sum += w[BULK ? ch * P : ch];                 // the carry
+        }
         if (sum != 0.f) atomicAdd(&norm_priv[(int64_t)slot * C * P + i], (double)sum);
     }
 }
