@@ -132,9 +132,8 @@ int grid_destroy(wg_grid* h)
     cudaFree(g.scratch);
     cudaFree(g.corr);
     cudaFree(g.icorr);
-    cudaFree(g.inv_norm);
-    if (g.plan_ok) cufftDestroy(g.plan);
-    if (g.plan_c_ok) cufftDestroy(g.plan_c);
+    for (cufftHandle plan : {g.plan_c2r, g.plan_r2c, g.plan_c2c})
+        if (plan >= 0) cufftDestroy(plan);
     delete h;
     return WG_OK;
 }

@@ -61,16 +61,13 @@ struct Grid {
     double* norm = nullptr;               // [n_chan][n_pol]
     unsigned long long* counters = nullptr;  // [8] accumulated statistics
     // grid_correct resources
-    float2* scratch = nullptr;            // [G][N][N][P], G = scratch_chans
+    float2* scratch = nullptr;            // planes of scratch_chans channels
     int scratch_chans = 0;
     double* corr = nullptr;               // [N] taper x sinc
     float* icorr = nullptr;               // [N] 1 / (taper x sinc)
-    float* inv_norm = nullptr;            // [n_chan][n_pol] 1 / N_p (0 where N_p = 0)
     int corr_s0 = -1, corr_beta = -1;
-    cufftHandle plan = 0;
-    cufftHandle plan_c = 0;               // batch of scratch_chans contiguous N x N planes
-    bool plan_c_ok = false;
-    bool plan_ok = false;
+    // cuFFT plans (-1: not made) of contiguous N x N planes: scratch_chans of them, scratch_chans x n_pol of them
+    cufftHandle plan_c2r = -1, plan_r2c = -1, plan_c2c = -1;
 };
 
 struct Table {
@@ -95,6 +92,7 @@ struct Table {
     std::vector<double> pswf;             // Legendre coefficients of psi_0 (even degrees)
     bool stacking = false;                // every plane holds the w = 0 kernel (w-stacking)
     std::vector<double> w_planes;         // w_k of each plane, wavelengths
+    float2* wplanes_d = nullptr;          // [K] the same, each as the sum of two floats
 };
 
 struct WorkList {

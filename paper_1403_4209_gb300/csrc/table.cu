@@ -221,26 +221,18 @@ int set_table_store(Table& t, int store)
 int free_table(Table& t)
 {
     cudaFree(t.data_lp);
-    t.data_lp = nullptr;
     cudaFree(t.pairs_lp);
     cudaFree(t.pairs);
-    cudaFree(t.poffsets_d);
-    t.pairs_lp = nullptr;
-    t.pairs = nullptr;
-    t.poffsets_d = nullptr;
     cudaFree(t.data);
-    cudaFree(t.zeta);
-    cudaFree(t.supports_d);
-    cudaFree(t.offsets_d);
-    cudaFree(t.wbounds_d);
-    cudaFree(t.wbounds_f);
-    cudaFree(t.zeta_f);
+    cudaFree(t.zeta);                              // the buffer of the small arrays
+    t.data_lp = t.pairs_lp = nullptr;
+    t.pairs = nullptr;
     t.data = nullptr;
-    t.zeta = nullptr;
+    t.zeta = t.wbounds_d = nullptr;
+    t.wplanes_d = nullptr;
     t.supports_d = t.offsets_d = nullptr;
-    t.wbounds_d = nullptr;
-    t.wbounds_f = nullptr;
-    t.zeta_f = nullptr;
+    t.poffsets_d = nullptr;
+    t.wbounds_f = t.zeta_f = nullptr;
     return WG_OK;
 }
 
@@ -260,22 +252,6 @@ static int finish_layout(Table& t)
     if (off >= (int64_t)1 << 31) return fail(WG_E_OOB_SUPPORT, "kernel table has %lld samples (limit 2^31)", (long long)off);
     t.n_samples = off;
     t.n_pairs = poff;
-    if (cudaMalloc(&t.data, sizeof(float2) * std::max<int64_t>(off, 1)) != cudaSuccess ||
-        cudaMalloc(&t.zeta, sizeof(double) * t.K * t.beta * t.beta) != cudaSuccess ||
-        cudaMalloc(&t.pairs, sizeof(float4) * std::max<int64_t>(poff, 1)) != cudaSuccess ||
-        cudaMalloc(&t.poffsets_d, sizeof(unsigned) * t.K) != cudaSuccess ||
-        cudaMalloc(&t.supports_d, sizeof(int) * t.K) != cudaSuccess ||
-        cudaMalloc(&t.offsets_d, sizeof(int) * t.K) != cudaSuccess ||
-        cudaMalloc(&t.wbounds_d, sizeof(double) * t.K) != cudaSuccess ||
-        cudaMalloc(&t.wbounds_f, sizeof(float) * t.K) != cudaSuccess ||
-        cudaMalloc(&t.zeta_f, sizeof(float) * t.K * t.beta * t.beta) != cudaSuccess) {
-        cudaGetLastError();
-        free_table(t);
-        return fail(WG_E_OOM, "cannot allocate the kernel table (%lld samples)", (long long)off);
-    }
-    WG_CUDA(cudaMemcpy(t.supports_d, t.supports.data(), sizeof(int) * t.K, cudaMemcpyHostToDevice));
-    WG_CUDA(cudaMemcpy(t.offsets_d, t.offsets.data(), sizeof(int) * t.K, cudaMemcpyHostToDevice));
-    WG_CUDA(cudaMemcpy(t.poffsets_d, poffsets.data(), sizeof(unsigned) * t.K, cudaMemcpyHostToDevice));
     // nearest plane in sqrt(w): plane k is chosen when b_k <= w < b_{k+1}, with
     // b_m = w_max (t t), t = (m - 1/2) / (K - 1), m = 1..K (b_K bounds the last plane)
     std::vector<double> wb(t.K, 0.0);
@@ -284,10 +260,41 @@ static int finish_layout(Table& t)
             const double tm = (m - 0.5) / (double)(t.K - 1);
             wb[m - 1] = t.w_max * (tm * tm);
         }
-    WG_CUDA(cudaMemcpy(t.wbounds_d, wb.data(), sizeof(double) * t.K, cudaMemcpyHostToDevice));
-    std::vector<float> wbf(t.K);
-    for (int m = 0; m < t.K; ++m) wbf[m] = (float)wb[m];     // round to nearest
-    WG_CUDA(cudaMemcpy(t.wbounds_f, wbf.data(), sizeof(float) * t.K, cudaMemcpyHostToDevice));
+    // the small arrays share one buffer and one copy: [zeta][wbounds][wplanes][supports][offsets][poffsets][wbounds_f][zeta_f]
+    const size_t K = t.K, nz = K * t.beta * t.beta;
+    const size_t bytes = sizeof(double) * (nz + 2 * K) + sizeof(int) * 4 * K + sizeof(float) * nz;
+    unsigned char* d = nullptr;
+    if (cudaMalloc(&t.data, sizeof(float2) * std::max<int64_t>(off, 1)) != cudaSuccess ||
+        cudaMalloc(&t.pairs, sizeof(float4) * std::max<int64_t>(poff, 1)) != cudaSuccess ||
+        cudaMalloc(&d, bytes) != cudaSuccess) {
+        cudaGetLastError();
+        free_table(t);
+        return fail(WG_E_OOM, "cannot allocate the kernel table (%lld samples)", (long long)off);
+    }
+    t.zeta = reinterpret_cast<double*>(d);
+    t.wbounds_d = t.zeta + nz;
+    t.wplanes_d = reinterpret_cast<float2*>(t.wbounds_d + K);
+    t.supports_d = reinterpret_cast<int*>(t.wplanes_d + K);
+    t.offsets_d = t.supports_d + K;
+    t.poffsets_d = reinterpret_cast<unsigned*>(t.offsets_d + K);
+    t.wbounds_f = reinterpret_cast<float*>(t.poffsets_d + K);
+    t.zeta_f = t.wbounds_f + K;
+    std::vector<unsigned char> h(sizeof(double) * 2 * K + sizeof(int) * 4 * K);
+    double* hw = reinterpret_cast<double*>(h.data());
+    float2* hp = reinterpret_cast<float2*>(hw + K);
+    int* hs = reinterpret_cast<int*>(hp + K);
+    unsigned* ho = reinterpret_cast<unsigned*>(hs + 2 * K);
+    float* hf = reinterpret_cast<float*>(ho + K);
+    for (size_t k = 0; k < K; ++k) {
+        const float hi = (float)t.w_planes[k];
+        hw[k] = wb[k];
+        hp[k] = make_float2(hi, (float)(t.w_planes[k] - (double)hi));
+        hs[k] = t.supports[k];
+        hs[K + k] = t.offsets[k];
+        ho[k] = poffsets[k];
+        hf[k] = (float)wb[k];                      // round to nearest
+    }
+    WG_CUDA(cudaMemcpy(t.wbounds_d, h.data(), h.size(), cudaMemcpyHostToDevice));
     return WG_OK;
 }
 
