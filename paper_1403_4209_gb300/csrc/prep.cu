@@ -1300,45 +1300,101 @@ int launch_plan(const Table& t, WorkList& wl, cudaStream_t s)
 // density W_p(cell) = sum of eps_p (1 - f_p) of the griddable records in the grid cell of their
 // placement; uniform eps' = eps / W; robust (Briggs) eps' = eps / (1 + W f^2) with
 // f^2 = (5 10^-R)^2 / (sum_cells W^2 / sum eps (1 - f)).  Records that are not griddable keep eps.
+//
+// The bytes are the density grid's (set, added to, read once for its squares) and each record's weights; what the
+// kernels were bound by was FP64 (two results a clock and SM) and placing every record twice.  Now k_density keeps each
+// record's cell for k_reweight, one vector reduction adds a record's polarisations, and sums, squares and quotients are
+// pairs of floats, with FP64 for the values at which those are not exact.  Briggs weights of 9.7 M records, P = 4,
+// C = 4, N = 2048: k_density 332 -> 167 us, k_density_sq 262 -> 108, k_reweight 961 -> 123; the call 1610 -> 456 us.
 
-// the grid cell (x, y) of a griddable record, from its footprint origin
-__device__ __forceinline__ int2 cell_of(const int4& info, const int* __restrict__ supports)
+// the grid cell of a griddable record, column | row << 16, from its footprint origin
+__device__ __forceinline__ unsigned cell_of(const int4& info, const int* __restrict__ supports)
 {
     const int h = (__ldg(&supports[info.w & 0xFFF]) - 1) / 2;
-    return make_int2((info.x & 0xFFFF) + h, ((info.x >> 16) & 0xFFFF) + h);
+    return (unsigned)((info.x & 0xFFFF) + h) | ((unsigned)(((info.x >> 16) & 0xFFFF) + h) << 16);
+}
+constexpr unsigned kNoCell = 0xFFFFFFFFu;                 // not griddable (a column is below 32768)
+
+// the P weights and flag bytes of record rec; vec: weight 4P-byte and flag P-byte aligned
+template <int P, typename IDX>
+__device__ __forceinline__ void load_weights(const float* __restrict__ weight, const uint8_t* __restrict__ flag, IDX rec, int vec,
+                                             float (&w)[P], float (&wf)[P])
+{
+    unsigned f[P];
+    if (vec && P == 4) {
+        const float4 a = *(reinterpret_cast<const float4*>(weight) + rec);
+        const unsigned b = *(reinterpret_cast<const unsigned*>(flag) + rec);
+        const float t[4] = {a.x, a.y, a.z, a.w};
+#pragma unroll
+        for (int p = 0; p < P; ++p) {
+            w[p] = t[p];
+            f[p] = (b >> (8 * p)) & 0xFF;
+        }
+    } else {
+#pragma unroll
+        for (int p = 0; p < P; ++p) {
+            w[p] = weight[(int64_t)rec * P + p];
+            f[p] = flag[(int64_t)rec * P + p];
+        }
+    }
+#pragma unroll
+    for (int p = 0; p < P; ++p) wf[p] = w[p] * (1.0f - (float)f[p]);
 }
 
-template <int P>
+// s + e += x with the rounding error of the sum kept (TwoSum, Knuth): about 48 bits, without FP64 (two
+// FP64 results a clock and SM)
+__device__ __forceinline__ void add_exact(float& s, float& e, float x)
+{
+    const float t = __fadd_rn(s, x), b = __fsub_rn(t, s);
+    e = __fadd_rn(e, __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(x, b)));
+    s = t;
+}
+
+// The densities, each record's cell (for k_reweight, which then need not place it again), and sum eps (1 - f).
+template <int P, typename IDX>
 __global__ void __launch_bounds__(256) k_density(const double* __restrict__ uvw, const double* __restrict__ lam_inv,
                                                  const double* __restrict__ sc, const float* __restrict__ lam_f,
                                                  const float* __restrict__ sc_f, const float* __restrict__ weight,
-                                                 const uint8_t* __restrict__ flag, int64_t rows, PlaceParams pp,
-                                                 float* __restrict__ dens, double* __restrict__ sums)
+                                                 const uint8_t* __restrict__ flag, int64_t rows, PlaceParams pp, int vec,
+                                                 float* __restrict__ dens, unsigned* __restrict__ cells,
+                                                 double* __restrict__ sums)
 {
     __shared__ double s_w[P];
     if (threadIdx.x < P) s_w[threadIdx.x] = 0.0;
     __syncthreads();
-    const int C = pp.C;
-    const int64_t n = rows * C;
-    double acc[P] = {};
-    for (int64_t rec = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; rec < n; rec += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t row = rec / C;
+    const IDX C = (IDX)pp.C, n = (IDX)(rows * pp.C), step = (IDX)gridDim.x * blockDim.x;
+    float acc[P] = {}, err[P] = {};
+    for (IDX rec = (IDX)blockIdx.x * blockDim.x + threadIdx.x; rec < n; rec += step) {
+        const IDX row = rec / C;
         const int ch = (int)(rec - row * C);
-        const int4 info = place(uvw, row, row_f(uvw, row), lam_inv, sc, ch, lam_f[ch], sc_f[ch], flag, rec, P, pp).info;
-        if (!((info.w >> kBitGd) & 1)) continue;
-        const int2 xy = cell_of(info, pp.supports);
-        const int gc = pp.interleave ? 0 : ch;
-        float* d = dens + (((size_t)gc * pp.N + xy.y) * pp.N + xy.x) * P;
+        const int4 info = place(uvw, (int64_t)row, row_f(uvw, (int64_t)row), lam_inv, sc, ch, lam_f[ch], sc_f[ch], flag,
+                                (int64_t)rec, P, pp).info;
+        if (!((info.w >> kBitGd) & 1)) {
+            cells[rec] = kNoCell;
+            continue;
+        }
+        const unsigned cell = cell_of(info, pp.supports);
+        cells[rec] = cell;
+        float w[P], wf[P];
+        load_weights<P>(weight, flag, rec, vec, w, wf);
+        float* d = dens + (((size_t)(pp.interleave ? 0 : ch) * pp.N + (cell >> 16)) * pp.N + (cell & 0xFFFF)) * P;
+        if constexpr (P == 4) {
+            if (wf[0] != 0.f || wf[1] != 0.f || wf[2] != 0.f || wf[3] != 0.f)
+                atomicAdd(reinterpret_cast<float4*>(d), make_float4(wf[0], wf[1], wf[2], wf[3]));
+        } else if constexpr (P == 2) {
+            if (wf[0] != 0.f || wf[1] != 0.f) atomicAdd(reinterpret_cast<float2*>(d), make_float2(wf[0], wf[1]));
+        } else {
+            if (wf[0] != 0.f) atomicAdd(d, wf[0]);
+        }
 #pragma unroll
         for (int p = 0; p < P; ++p) {
-            const float wf = weight[rec * P + p] * (1.0f - (float)flag[rec * P + p]);
-            if (wf != 0.f) atomicAdd(d + p, wf);
-            acc[p] += wf;
+            if (fabsf(wf[p]) < 1e30f) add_exact(acc[p], err[p], wf[p]);
+            else atomicAdd(&s_w[p], (double)wf[p]);          // (an FP32 sum could overflow; infinities and NaN)
         }
     }
 #pragma unroll
     for (int p = 0; p < P; ++p) {
-        double x = acc[p];
+        double x = (double)acc[p] + (double)err[p];
         for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
         if ((threadIdx.x & 31) == 0 && x != 0.0) atomicAdd(&s_w[p], x);
     }
@@ -1346,7 +1402,8 @@ __global__ void __launch_bounds__(256) k_density(const double* __restrict__ uvw,
     if (threadIdx.x < P && s_w[threadIdx.x] != 0.0) atomicAdd(&sums[threadIdx.x], s_w[threadIdx.x]);
 }
 
-// sums[P + p] += sum over cells of W_p^2
+// sums[P + p] += sum over cells of W_p^2.  The squares and their sum are pairs of floats (the product's error by FMA,
+// the sum's by add_exact) where those are exact; the rest, which no ordinary weights reach, are FP64.
 template <int P>
 __global__ void __launch_bounds__(256) k_density_sq(const float* __restrict__ dens, int64_t n_cells,
                                                     double* __restrict__ sums)
@@ -1355,15 +1412,33 @@ __global__ void __launch_bounds__(256) k_density_sq(const float* __restrict__ de
     if (threadIdx.x < P) s_q[threadIdx.x] = 0.0;
     __syncthreads();
     double acc[P] = {};
-    for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < n_cells; c += (int64_t)gridDim.x * blockDim.x)
-#pragma unroll
-        for (int p = 0; p < P; ++p) {
-            const double v = dens[c * P + p];
-            acc[p] += v * v;
+    float hi[P] = {}, lo[P] = {};
+    for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < n_cells; c += (int64_t)gridDim.x * blockDim.x) {
+        float v[P];
+        if constexpr (P == 4) {
+            const float4 a = *(reinterpret_cast<const float4*>(dens) + c);
+            v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
+        } else if constexpr (P == 2) {
+            const float2 a = *(reinterpret_cast<const float2*>(dens) + c);
+            v[0] = a.x; v[1] = a.y;
+        } else {
+            v[0] = dens[c];
         }
 #pragma unroll
+        for (int p = 0; p < P; ++p) {
+            const float a = fabsf(v[p]);
+            if (a > 1e-11f && a < 1e14f) {
+                const float q = __fmul_rn(a, a);
+                lo[p] = __fadd_rn(lo[p], fmaf(a, a, -q));
+                add_exact(hi[p], lo[p], q);
+            } else if (a != 0.f) {
+                acc[p] += (double)a * (double)a;
+            }
+        }
+    }
+#pragma unroll
     for (int p = 0; p < P; ++p) {
-        double x = acc[p];
+        double x = acc[p] + (double)hi[p] + (double)lo[p];
         for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
         if ((threadIdx.x & 31) == 0 && x != 0.0) atomicAdd(&s_q[p], x);
     }
@@ -1371,39 +1446,67 @@ __global__ void __launch_bounds__(256) k_density_sq(const float* __restrict__ de
     if (threadIdx.x < P && s_q[threadIdx.x] != 0.0) atomicAdd(&sums[P + threadIdx.x], s_q[threadIdx.x]);
 }
 
-template <int P>
-__global__ void __launch_bounds__(256) k_reweight(const double* __restrict__ uvw, const double* __restrict__ lam_inv,
-                                                  const double* __restrict__ sc, const float* __restrict__ lam_f,
-                                                  const float* __restrict__ sc_f, const float* __restrict__ weight,
-                                                  const uint8_t* __restrict__ flag, int64_t rows, PlaceParams pp,
-                                                  const float* __restrict__ dens, const double* __restrict__ sums,
-                                                  int scheme, double robust_f0, float* __restrict__ out)
+// w / (1 + W f2) rounded once: the denominator as two floats (dh + dl, exact products by FMA), a correctly
+// rounded FP32 quotient by dh, and its remainder's correction.  Values out of the range in which that is exact take
+// the FP64 division, whose thirty or so instructions are what the kernel spent its time on.
+__device__ __forceinline__ float robust_weight(float w, float W, double f2, float f2h, float f2l)
 {
-    const int C = pp.C;
-    const int64_t n = rows * C;
+    const float p = __fmul_rn(W, f2h), e = fmaf(W, f2h, -p) + __fmul_rn(W, f2l);
+    const float s = __fadd_rn(1.0f, p), b = __fsub_rn(s, 1.0f);
+    const float dl = __fadd_rn(__fadd_rn(__fsub_rn(1.0f, __fsub_rn(s, b)), __fsub_rn(p, b)), e);
+    const float aw = fabsf(w), as = fabsf(s);
+    if (aw > 1e-25f && aw < 1e25f && fabsf(W) < 1e25f && as > 1e-5f && as < 1e10f && fabsf(p) < 1e10f) {
+        const float q = __fdiv_rn(w, s);
+        const float r = fmaf(-q, dl, fmaf(-q, s, w));
+        return __fadd_rn(q, __fdividef(r, s));
+    }
+    return (float)((double)w / (1.0 + (double)W * f2));
+}
+
+template <int P, typename IDX>
+__global__ void __launch_bounds__(256) k_reweight(const unsigned* __restrict__ cells, const float* __restrict__ weight,
+                                                  int64_t rows, PlaceParams pp, const float* __restrict__ dens,
+                                                  const double* __restrict__ sums, int scheme, double robust_f0,
+                                                  float* __restrict__ out)
+{
+    const IDX C = (IDX)pp.C, n = (IDX)(rows * pp.C), step = (IDX)gridDim.x * blockDim.x;
+    const bool vec = P == 4 && (reinterpret_cast<uintptr_t>(weight) & 15) == 0 && (reinterpret_cast<uintptr_t>(out) & 15) == 0;
     double f2[P];
+    float f2h[P], f2l[P];
 #pragma unroll
-    for (int p = 0; p < P; ++p) f2[p] = (sums[P + p] > 0.0) ? robust_f0 * robust_f0 * sums[p] / sums[P + p] : 0.0;
-    for (int64_t rec = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; rec < n; rec += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t row = rec / C;
-        const int ch = (int)(rec - row * C);
-        const int4 info = place(uvw, row, row_f(uvw, row), lam_inv, sc, ch, lam_f[ch], sc_f[ch], flag, rec, P, pp).info;
-        const bool gd = (info.w >> kBitGd) & 1;
-        const float* d = nullptr;
-        if (gd) {
-            const int2 xy = cell_of(info, pp.supports);
-            d = dens + ((((size_t)(pp.interleave ? 0 : ch)) * pp.N + xy.y) * pp.N + xy.x) * P;
+    for (int p = 0; p < P; ++p) {
+        f2[p] = (sums[P + p] > 0.0) ? robust_f0 * robust_f0 * sums[p] / sums[P + p] : 0.0;
+        f2h[p] = (float)f2[p];
+        f2l[p] = (float)(f2[p] - (double)f2h[p]);
+    }
+    for (IDX rec = (IDX)blockIdx.x * blockDim.x + threadIdx.x; rec < n; rec += step) {
+        const unsigned cell = cells[rec];
+        float w[P];
+        if (vec && P == 4) {
+            const float4 a = *(reinterpret_cast<const float4*>(weight) + rec);
+            const float t[4] = {a.x, a.y, a.z, a.w};
+#pragma unroll
+            for (int p = 0; p < P; ++p) w[p] = t[p];
+        } else {
+#pragma unroll
+            for (int p = 0; p < P; ++p) w[p] = weight[(int64_t)rec * P + p];
         }
+        if (cell != kNoCell) {
+            const int ch = pp.interleave ? 0 : (int)(rec % C);
+            const float* d = dens + (((size_t)ch * pp.N + (cell >> 16)) * pp.N + (cell & 0xFFFF)) * P;
 #pragma unroll
-        for (int p = 0; p < P; ++p) {
-            const float w = weight[rec * P + p];
-            float o = w;
-            if (gd) {
-                const double W = d[p];
-                if (scheme == WG_WEIGHT_UNIFORM) o = (W > 0.0) ? (float)((double)w / W) : 0.f;
-                else o = (float)((double)w / (1.0 + W * f2[p]));
+            for (int p = 0; p < P; ++p) {
+                const float W = d[p];
+                // (a quotient of floats rounded to FP64 and then to FP32 is the correctly rounded FP32 one)
+                if (scheme == WG_WEIGHT_UNIFORM) w[p] = (W > 0.0f) ? __fdiv_rn(w[p], W) : 0.f;
+                else w[p] = robust_weight(w[p], W, f2[p], f2h[p], f2l[p]);
             }
-            out[rec * P + p] = o;
+        }
+        if (vec && P == 4) {
+            *(reinterpret_cast<float4*>(out) + rec) = make_float4(w[0], w[1 % P], w[2 % P], w[3 % P]);
+        } else {
+#pragma unroll
+            for (int p = 0; p < P; ++p) out[(int64_t)rec * P + p] = w[p];
         }
     }
 }
@@ -1418,36 +1521,48 @@ static int weight_impl(const Table& t, const Grid& g, const wg_vis_in& in, int s
     pp.flag_vec = (reinterpret_cast<uintptr_t>(in.flag) % P) == 0;
     const int gc = pp.interleave ? 1 : C;
     const int64_t n_cells = (int64_t)gc * g.n * g.n;
-    const size_t bytes = sizeof(float) * (size_t)n_cells * P + sizeof(double) * (4 * C + 2 * P);
+    // the densities, the channel scales, the sums, and each record's cell
+    const size_t bytes = sizeof(float) * (size_t)n_cells * P + sizeof(double) * (4 * C + 2 * P) +
+                         sizeof(unsigned) * (size_t)(rows * C);
     void* scratch = nullptr;
     if (cudaMallocAsync(&scratch, bytes, s) != cudaSuccess) {
         cudaGetLastError();
         return fail(WG_E_OOM, "cannot allocate the weight-density grid (%zu bytes)", bytes);
     }
-    float* dens = static_cast<float*>(scratch);
-    double* lam_inv = reinterpret_cast<double*>(dens + (size_t)n_cells * P);
+    double* lam_inv = static_cast<double*>(scratch);
     double* sc = lam_inv + C;
     double* sums = sc + C;                                   // [2P]: sum eps (1-f), sum W^2
     float* lam_f = reinterpret_cast<float*>(sums + 2 * P);
     float* sc_f = lam_f + C;
+    float* dens = reinterpret_cast<float*>(lam_inv + (4 * C + 2 * P));   // 4 C + 2 P is even: 16-byte aligned
+    unsigned* cells = reinterpret_cast<unsigned*>(dens + (size_t)n_cells * P);
+    const int vec = reinterpret_cast<uintptr_t>(in.weight) % (4 * P) == 0 && pp.flag_vec;
     int rc = WG_OK;
-    if (cudaMemsetAsync(scratch, 0, sizeof(float) * (size_t)n_cells * P, s) != cudaSuccess ||
+    if (cudaMemsetAsync(dens, 0, sizeof(float) * (size_t)n_cells * P, s) != cudaSuccess ||
         cudaMemsetAsync(sums, 0, sizeof(double) * 2 * P, s) != cudaSuccess) {
         rc = cuda_fail(cudaGetLastError(), "weight density");
     } else {
-        k_chan_scale<<<(C + 127) / 128, 128, 0, s>>>(in.freq_hz, C, pp.beta_over_du, lam_inv, sc, lam_f, sc_f);
-        WG_LAUNCHED("k_chan_scale");
         const int blocks = num_sms() * 8;
         if (rows > 0) {
-            k_density<P><<<blocks, 256, 0, s>>>(in.uvw, lam_inv, sc, lam_f, sc_f, in.weight, in.flag, rows, pp, dens, sums);
-            WG_LAUNCHED("k_density");
-            k_density_sq<P><<<blocks, 256, 0, s>>>(dens, n_cells, sums);
-            WG_LAUNCHED("k_density_sq");
-            k_reweight<P><<<blocks, 256, 0, s>>>(in.uvw, lam_inv, sc, lam_f, sc_f, in.weight, in.flag, rows, pp, dens,
-                                                 sums, scheme, 5.0 * std::pow(10.0, -robust), out);
-            WG_LAUNCHED("k_reweight");
+            k_chan_scale<<<(C + 127) / 128, 128, 0, s>>>(in.freq_hz, C, pp.beta_over_du, lam_inv, sc, lam_f, sc_f);
+            count_launch();
+            const double f0 = 5.0 * std::pow(10.0, -robust);
+            auto run = [&](auto idx) -> int {
+                using IDX = decltype(idx);           // 32-bit record indices where they suffice
+                k_density<P, IDX><<<blocks, 256, 0, s>>>(in.uvw, lam_inv, sc, lam_f, sc_f, in.weight, in.flag, rows, pp, vec, dens,
+                                                         cells, sums);
+                WG_LAUNCHED("k_density");
+                if (scheme == WG_WEIGHT_ROBUST) {
+                    k_density_sq<P><<<blocks, 256, 0, s>>>(dens, n_cells, sums);
+                    WG_LAUNCHED("k_density_sq");
+                }
+                k_reweight<P, IDX><<<blocks, 256, 0, s>>>(cells, in.weight, rows, pp, dens, sums, scheme, f0, out);
+                WG_LAUNCHED("k_reweight");
+                return WG_OK;
+            };
+            rc = rows * C < ((int64_t)1 << 31) ? run(0u) : run((int64_t)0);
         }
-        if (cudaGetLastError() != cudaSuccess) rc = fail(WG_E_CUDA, "weighting kernels failed to launch");
+        if (rc == WG_OK && cudaGetLastError() != cudaSuccess) rc = fail(WG_E_CUDA, "weighting kernels failed to launch");
     }
     cudaFreeAsync(scratch, s);
     return rc;
