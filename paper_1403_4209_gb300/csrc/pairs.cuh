@@ -104,7 +104,9 @@ struct TaskParams {
     const int4* entries;
     const float2* gamma;
     const int* seg_off;
+    const int* seg_nblk;
     const long long* scal;
+    const long long* n_tasks;
     const int* supports;
     const int* offsets;          // C-1 offset of each plane (entries' z refer to it)
     const unsigned* poffsets;    // first pair of each plane in the paired table
@@ -190,6 +192,15 @@ __device__ __forceinline__ unsigned move_classes(unsigned (&toff)[NU], const int
         wraps |= w ? 1u << u : 0u;
     }
     return wraps;
+}
+
+// Places a pair of class cl (column | row << 16) in the footprint of entry E: its column and row there.
+__device__ __forceinline__ int2 place_class(int cl, const Staged& E, int S, int H)
+{
+    int du = (cl & 0xFFFF) + (E.y & 0xFFFF), dv = (cl >> 16) + (E.y >> 16);
+    du -= (du >= S) ? S : 0;
+    dv -= (dv >= H) ? H : 0;
+    return make_int2(du, dv);
 }
 
 constexpr int kPartMin = 4;   // entries of the shortest part of a segment
@@ -336,11 +347,12 @@ struct Chunk {
 // segment is cut into parts, so that every warp has something to do (17 tasks on 2432 warps: 204 -> 25 us).
 struct Item {
     int blk, e0, n;          // block of the footprint, first entry, entries
+    int seg;                 // its segment
 };
 
 __device__ __forceinline__ int item_parts(const TaskParams& tp)
 {
-    const long long n_tasks = tp.scal[1], warps = (long long)gridDim.x * (blockDim.x >> 5);
+    const long long n_tasks = *tp.n_tasks, warps = (long long)gridDim.x * (blockDim.x >> 5);
     if (n_tasks <= 0 || n_tasks >= warps) return 1;
     return (int)min((long long)(tp.seg_len / kPartMin), (warps + n_tasks - 1) / n_tasks);
 }
@@ -352,7 +364,7 @@ __device__ __forceinline__ bool next_item(const TaskParams& tp, int parts, int l
     if (lane == 0) w = atomicAdd(tp.counter, 1u);
     w = __shfl_sync(0xffffffffu, w, 0);
     const unsigned t = parts > 1 ? w / (unsigned)parts : w;
-    if ((long long)t >= tp.scal[1]) return false;
+    if ((long long)t >= *tp.n_tasks) return false;
     // the task's segment: each step probes 32 places
     int lo = 0, hi = (int)tp.scal[2];
     while (hi - lo > 1) {
@@ -362,6 +374,7 @@ __device__ __forceinline__ bool next_item(const TaskParams& tp, int parts, int l
         hi = min(hi, lo + step);
     }
     it.blk = (int)t - __ldg(&tp.seg_off[lo]);
+    it.seg = lo;
     it.e0 = lo * tp.seg_len;
     it.n = (int)min((long long)tp.seg_len, tp.scal[0] - it.e0);
     if (parts > 1) {
@@ -373,9 +386,10 @@ __device__ __forceinline__ bool next_item(const TaskParams& tp, int parts, int l
     return true;
 }
 
-inline TaskParams task_params(const Grid& g, const Table& t, const WorkList& wl, unsigned* counter)
+// jumps: the tasks of the segments whose footprints jump about, not all
+inline TaskParams task_params(const Grid& g, const Table& t, const WorkList& wl, unsigned* counter, bool jumps)
 {
-    return {wl.entries, wl.gamma, wl.seg_off,    wl.scal, t.supports_d, t.offsets_d, t.poffsets_d, g.n,     t.K,
+    return {wl.entries, wl.gamma, jumps ? wl.seg_offj : wl.seg_off, wl.seg_nblk, wl.scal, wl.scal + (jumps ? 4 : 1), t.supports_d, t.offsets_d, t.poffsets_d, g.n,     t.K,
             g.n_chan,    t.beta * t.beta, t.n_samples, wl.seg_len,   wl.slots,    counter,      wl.scal + 3};
 }
 
