@@ -210,7 +210,7 @@ def measured_ceilings(real_rate: float, P: int) -> dict:
             "frac_of_fma": round(real_rate / fma, 4), "frac_of_fetch_l2": round(real_rate / l2, 4),
             "frac_of_min": round(real_rate / low, 4),
             "note": "real gridder updates/s against measured ceilings; kernel samples stream mostly from L2 "
-                    "(ncu l1tex hit rate about 16 %), so the fetch ceiling is the L2 one"}
+                    "(ncu l1tex hit rate about 8 %), so the fetch ceiling is the L2 one"}
 
 
 def _gridder_traffic(per_launch_units):

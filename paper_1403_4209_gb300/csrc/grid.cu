@@ -6,6 +6,7 @@
 // kUnitsMax point pairs of the footprint by their class (pairs.cuh), so lanes never touch the same
 // pixel and accumulate in registers while the pair stays the same; when it moves, the lane flushes
 // its accumulators with vector FP32 atomics (all polarisations of a pixel are contiguous).
+// Segments whose footprints mostly jump are left to k_grid_jumps.
 //
 // What bounds it: instruction issue and the FMA pipe (59 % and 50 % busy at four polarisations, 128
 // registers, 16 warps an SM), then the L1 data path (68 %: every sample is used once per entry and comes from L2).
@@ -208,11 +209,15 @@ __device__ __noinline__ void slow_entry(const float2* g, int S, int unit0, int u
 
 }  // namespace
 
-template <int P, typename TS, bool COMP>
-__global__ void __launch_bounds__(kWarps * 32, P == 4 ? 4 : P == 2 ? 5 : 7) k_grid(TaskParams tp,
-                                                                                  const char* __restrict__ table,
-                                                                                  float2* __restrict__ grid,
-                                                                                  float2* __restrict__ errgrid)
+// SMALL: every support of the table has at most kSmallPairs pairs, two units (up to support 9).  Two units a lane leave
+// registers for five blocks an SM, and none idle: support 7 at P = 4 from 387 to 226 us, support 9 from 409 to 241,
+// compensated from 713 to 551 (single points took 281, 332 and 666).
+constexpr int kSmallPairs = 64;
+template <int P, typename TS, bool COMP, bool SMALL>
+__global__ void __launch_bounds__(kWarps * 32, P == 4 ? (SMALL ? 5 : 4) : P == 2 ? 5 : 7) k_grid(TaskParams tp,
+                                                                                                const char* __restrict__ table,
+                                                                                                float2* __restrict__ grid,
+                                                                                                float2* __restrict__ errgrid)
 {
     __shared__ __align__(16) unsigned char smem[kWarps * Chunk<P, true>::kBytes];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -258,7 +263,7 @@ __global__ void __launch_bounds__(kWarps * 32, P == 4 ? 4 : P == 2 ? 5 : 7) k_gr
                 // the variant for small supports saves idle units at one and two polarisations (28 against 33 us on
                 // 127 k entries of support 7); at four, and with compensation, its code costs more in the
                 // instruction cache (21.1 against 20.5 ms on 21 M entries of supports 9..65)
-                if (P == 4 || COMP || un.y - un.x > 2)
+                if (!SMALL && (P == 4 || COMP || un.y - un.x > 2))
                     j = run_entries<P, TS, COMP, kUnitsMax>(ck, j, S, ch, un, tp, report, table, grid, errgrid);
                 else
                     j = run_entries<P, TS, COMP, 2>(ck, j, S, ch, un, tp, report, table, grid, errgrid);
@@ -442,20 +447,20 @@ __global__ void k_fold(float4* __restrict__ grid, float4* __restrict__ err, int6
     err[i] = make_float4(0.f, 0.f, 0.f, 0.f);
 }
 
-template <int P, typename TS, bool COMP>
+template <int P, typename TS, bool COMP, bool SMALL>
 static int grid_launch(Grid& g, const Table& t, const WorkList& wl, const void* table, const AccumulateParams& acc,
                        cudaStream_t s)
 {
     static int blocks_per_sm = 0, jump_blocks = 0;
     if (blocks_per_sm == 0 &&
-        (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks_per_sm, k_grid<P, TS, COMP>, kWarps * 32, 0) != cudaSuccess ||
+        (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks_per_sm, k_grid<P, TS, COMP, SMALL>, kWarps * 32, 0) != cudaSuccess ||
          blocks_per_sm < 1))
         blocks_per_sm = 1;
     if (jump_blocks == 0 &&
         (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&jump_blocks, k_grid_jumps<P, TS, COMP>, kWarps * 32, 0) != cudaSuccess ||
          jump_blocks < 1))
         jump_blocks = 1;
-    k_grid<P, TS, COMP><<<num_sms() * blocks_per_sm, kWarps * 32, 0, s>>>(
+    k_grid<P, TS, COMP, SMALL><<<num_sms() * blocks_per_sm, kWarps * 32, 0, s>>>(
         task_params(g, t, wl, wl.task_counter + 2, false), static_cast<const char*>(table), g.data, g.err);
     WG_LAUNCHED("k_grid");
     k_grid_jumps<P, TS, COMP><<<num_sms() * jump_blocks, kWarps * 32, 0, s>>>(
@@ -464,14 +469,22 @@ static int grid_launch(Grid& g, const Table& t, const WorkList& wl, const void* 
     return WG_OK;
 }
 
+template <int P, bool COMP, bool SMALL>
+static int grid_store(Grid& g, const Table& t, const WorkList& wl, const AccumulateParams& acc, cudaStream_t s)
+{
+    switch (t.store) {
+        case WG_BF16: return grid_launch<P, __nv_bfloat162, COMP, SMALL>(g, t, wl, t.pairs_lp, acc, s);
+        case WG_F16: return grid_launch<P, __half2, COMP, SMALL>(g, t, wl, t.pairs_lp, acc, s);
+        default: return grid_launch<P, float2, COMP, SMALL>(g, t, wl, t.pairs, acc, s);
+    }
+}
+
 template <int P, bool COMP>
 static int grid_dispatch(Grid& g, const Table& t, const WorkList& wl, const AccumulateParams& acc, cudaStream_t s)
 {
-    switch (t.store) {
-        case WG_BF16: return grid_launch<P, __nv_bfloat162, COMP>(g, t, wl, t.pairs_lp, acc, s);
-        case WG_F16: return grid_launch<P, __half2, COMP>(g, t, wl, t.pairs_lp, acc, s);
-        default: return grid_launch<P, float2, COMP>(g, t, wl, t.pairs, acc, s);
-    }
+    if constexpr (P == 4)          // (at fewer polarisations k_grid has the two-unit loop beside the other)
+        if (t.max_support * ((t.max_support + 1) / 2) <= kSmallPairs) return grid_store<P, COMP, true>(g, t, wl, acc, s);
+    return grid_store<P, COMP, false>(g, t, wl, acc, s);
 }
 
 template <int P>

@@ -9,6 +9,7 @@ import torch
 import oracle
 import paper_1403_4209_gb300 as wg
 from gpu_common import max_rel, rel_l2
+from test_gpu_pairs import _case as _walk_case
 from test_gpu_pairs import _grid, _tables
 
 pytestmark = pytest.mark.gpu
@@ -70,3 +71,14 @@ def test_nonfinite_among_jumps(P):
     pl0 = oracle.place(batch.uvw.cpu().numpy(), batch.freq.cpu().numpy(), 1.0, N, ref, flag=fl)
     want = oracle.grid_plain(pl0, ref, vis, wt, fl, N)[0, ..., 0]
     assert np.abs(g[..., 0][~hit] - want[~hit]).max() < 1e-5 * np.abs(want).max()
+
+
+@pytest.mark.parametrize("supports", [[9], [1, 5, 9]], ids=str)
+def test_tables_of_two_units(supports):
+    # P = 4 with every support at most 9: the two-unit kernel, at its largest support (45 pairs)
+    N = 60
+    ref, tab, pl, batch, vis, wt, fl = _walk_case(supports, 4, N, 3000, 21, C=2)
+    want = oracle.grid_plain(pl, ref, vis, wt, fl, N)
+    for plan, comp in ((None, False), ((32, 64, False), False), ((256, 256, True), True)):
+        got = _grid(tab, batch, 4, N, 2, plan, comp)[0].data.cpu().numpy()
+        assert rel_l2(got, want) < 1e-5 and max_rel(got, want) < 1e-5
