@@ -126,7 +126,7 @@ typedef int4 Staged;
 // A move of the footprint by one column or row: every pair's sample offset (in pairs) shifts by x; the
 // one class column (or row) that left the footprint wraps to the other side, its offset shifts by y;
 // z: what is added to a wrapped pair's first pixel (column | row << 16);
-// w: the class | the byte selector of its axis in a packed class << 16.
+// w: the class | the byte selector of its axis in a packed class << 16; -1 (the degridder's): a jump.
 typedef int4 Move;
 __device__ __forceinline__ int key_support(int key) { return key >> 16; }
 __device__ __forceinline__ int key_chan(int key) { return key & 0xFFFF; }
@@ -234,7 +234,8 @@ struct Chunk {
     int (*cur)[32];          // [kUnitsMax][32] the first pixels of the pairs they hold
     int lane;
     int e0, left, cnt;       // the chunk's first entry in the lists, entries from there to the item's end, its entries
-    unsigned kc;             // entries that start a run: another support or channel, a jump, or around a slow one
+    unsigned kc;             // entries that start a run: another support or channel, a jump (of the gridder's), or around
+                             // a slow one
     unsigned mv;             // entries whose footprint differs from their predecessor's (and kc)
     unsigned slow;           // entries with an infinite or NaN visibility
 
@@ -319,12 +320,13 @@ struct Chunk {
         const int cn = along_x ? s.y & 0xFFFF : s.y >> 16;                 // (-origin) mod md
         const int o = cn ? md - cn : 0;                                    // origin mod md
         const int c = d > 0 ? (o ? o - 1 : md - 1) : o;                    // the class that wraps
-        const bool k = s.w != qk || sl || qs || abs(dx) + abs(dy) > 1;
+        const bool far = abs(dx) + abs(dy) > 1;
+        const bool k = s.w != qk || sl || qs || (GAMMA && far);
         kc = __ballot_sync(0xffffffffu, in && k);
         mv = __ballot_sync(0xffffffffu, in && (k || s.x != qf));
         e[lane] = s;
         m[lane] = make_int4(-d * step, d * (md - 1) * step, along_x ? d * S : d * H * 65536,
-                            c | ((along_x ? 0x4410 : 0x4432) << 16));
+                            !GAMMA && far ? -1 : c | ((along_x ? 0x4410 : 0x4432) << 16));
         z[lane] = (unsigned)s.z;
         if constexpr (GAMMA) {
 #pragma unroll

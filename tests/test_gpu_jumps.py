@@ -82,3 +82,18 @@ def test_tables_of_two_units(supports):
     for plan, comp in ((None, False), ((32, 64, False), False), ((256, 256, True), True)):
         got = _grid(tab, batch, 4, N, 2, plan, comp)[0].data.cpu().numpy()
         assert rel_l2(got, want) < 1e-5 and max_rel(got, want) < 1e-5
+
+
+@pytest.mark.parametrize("kind", ["few", "half", "any", "mixed"])
+@pytest.mark.parametrize("P", [1, 2, 4])
+@pytest.mark.parametrize("supports", [[1], [7], [9, 15], [31, 45]], ids=str)
+def test_degridding_lists_of_jumps(supports, P, kind):
+    ref, tab, pl, batch, vis, wt, fl, N = _case(kind, supports, P, 900, 13 * P + len(kind))
+    rng = np.random.default_rng(P)
+    y = (rng.normal(size=(1, N, N, P)) + 1j * rng.normal(size=(1, N, N, P))).astype(np.complex64)
+    want = oracle.degrid(pl, ref, y.astype(np.complex128), wt, fl)
+    for plan in (None, (32, 64, False), (256, 256, True)):
+        g, work = _grid(tab, batch, P, N, 1, plan)
+        g.data.copy_(torch.as_tensor(y))
+        got = wg.degrid_vis(g, tab, batch, work).cpu().numpy().reshape(-1, P)
+        assert max_rel(got, want) < 1e-5
