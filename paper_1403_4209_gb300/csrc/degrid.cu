@@ -344,7 +344,8 @@ __global__ void __launch_bounds__(kWarps * 32, P == 4 ? 4 : 5) k_degrid_sum(Task
 // One block per preparation tile (rpb rows x all channels) writes the tile's output records
 // row-major.  Phase 1 puts each entry's sums into the shared-memory tile at the records of its
 // run that fall in the tile (the run before the tile's first head of a list can reach into
-// it), phase 2 stores the tile with coalesced vector stores, conjugated back where psi = -1
+// it), phase 2 stores the tile with coalesced stores (vec: out is 16-byte aligned, two
+// polarisations a store; callers need only align it to a polarisation's 8 bytes), conjugated back where psi = -1
 // (the take-conjugate class bit), with the cross hands swapped back under cross-hand swapping,
 // and for the adjoint mode scaled by eps (1 - f).  Records that are not griddable are in no run
 // and keep the tile's zero.  Lists: one per input channel (rows), or one in natural record
@@ -354,7 +355,7 @@ __global__ void __launch_bounds__(512) k_degrid_tile(const int2* __restrict__ ru
                                                      const int* __restrict__ tile_off, const int* __restrict__ chan_base,
                                                      const uint8_t* __restrict__ rclass, const float* __restrict__ weight,
                                                      const uint8_t* __restrict__ flag, int adjoint, int cross_swap,
-                                                     int interleave, int64_t rows, int rpb, int C, int64_t n_tiles,
+                                                     int interleave, int vec, int64_t rows, int rpb, int C, int64_t n_tiles,
                                                      float2* __restrict__ out)
 {
     extern __shared__ __align__(16) float2 s_out[];      // [rpb * C][P]
@@ -406,12 +407,13 @@ __global__ void __launch_bounds__(512) k_degrid_tile(const int2* __restrict__ ru
             }
         }
         float2* o = out + rec * P;
-        if constexpr (P == 1) {
-            o[0] = v[0];
+        if (P == 1 || !vec) {
+#pragma unroll
+            for (int p = 0; p < P; ++p) o[p] = v[p];
         } else {
 #pragma unroll
             for (int h = 0; h < P; h += 2)
-                *reinterpret_cast<float4*>(o + h) = make_float4(v[h].x, v[h].y, v[h + 1].x, v[h + 1].y);
+                *reinterpret_cast<float4*>(o + h) = make_float4(v[h].x, v[h].y, v[(h + 1) % P].x, v[(h + 1) % P].y);
         }
     }
 }
@@ -456,7 +458,8 @@ static int degrid_impl(const Grid& g, const Table& t, const wg_vis_in& in, const
     if (wl.n_tiles == 0) return WG_OK;     // no records
     k_degrid_tile<P><<<(unsigned)wl.n_tiles, 512, tile_smem, s>>>(
         wl.runs, wl.dacc, wl.tile_cnt, wl.chan_base, wl.rclass, in.weight, in.flag, mode == WG_DEGRID_ADJOINT ? 1 : 0,
-        wl.cross_swap ? 1 : 0, wl.interleave ? 1 : 0, in.n_rows, wl.rpb, in.n_chan, wl.n_tiles, out);
+        wl.cross_swap ? 1 : 0, wl.interleave ? 1 : 0, reinterpret_cast<uintptr_t>(out) % 16 == 0 ? 1 : 0,
+        in.n_rows, wl.rpb, in.n_chan, wl.n_tiles, out);
     WG_LAUNCHED("k_degrid_tile");
     return WG_OK;
 }
