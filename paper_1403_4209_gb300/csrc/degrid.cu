@@ -6,9 +6,9 @@
 //
 // k_degrid_sum runs the gridder's tasks (a segment of consecutive entries x one block of the
 // footprint, as the work list's plan defines them) on the gridder's point pairs and ownership
-// (pairs.cuh).  A lane keeps its pairs' pixel values in registers and reloads a pair only when the
-// footprint moves and the class's pixels change; for consecutive entries of a track that keep the footprint and
-// differ only in the sub-kernel it loads nothing but the kernel samples.  Per entry each lane sums its
+// (pairs.cuh).  A lane keeps its pairs' pixel values in registers; when the footprint moves, by one column or
+// anywhere, its pairs are placed anew and the pixels that they did not hold are loaded.  For consecutive entries of a track
+// that keep the footprint and differ only in the sub-kernel it loads nothing but the kernel samples.  Per entry each lane sums its
 // pairs into 2P floats; these go through a shared-memory transpose (batches of 64 / (2P)
 // entries), after which each lane holds two components of one entry summed over the warp and
 // adds them to a per-entry FP32 accumulator with one vector atomic per footprint block.  It is bound like
@@ -32,18 +32,18 @@ constexpr int kWarps = 4;           // warps per block of k_degrid_sum
 constexpr int kTileCap = 4096;      // records per preparation tile: rpb x C <= max(kTileRecords, n_chan <= 4096)
 static_assert(kTileRecords <= kTileCap, "a preparation tile must fit the degridder's output tile");
 
-// the P polarisations of one pixel
+// the P polarisations of one pixel, each (re, im) as it is stored
 template <int P>
-__device__ __forceinline__ void load_pixel(const float2* __restrict__ g, float2 (&v)[P])
+__device__ __forceinline__ void load_pixel(const float2* __restrict__ g, f32x2 (&v)[P])
 {
     if constexpr (P == 1) {
-        v[0] = __ldg(g);
+        v[0] = __ldg(reinterpret_cast<const f32x2*>(g));
     } else {
 #pragma unroll
         for (int h = 0; h < P; h += 2) {
-            const float4 a = __ldg(reinterpret_cast<const float4*>(g + h));
-            v[h] = make_float2(a.x, a.y);
-            v[h + 1] = make_float2(a.z, a.w);
+            const ulonglong2 a = __ldg(reinterpret_cast<const ulonglong2*>(g + h));
+            v[h] = a.x;
+            v[h + 1] = a.y;
         }
     }
 }
@@ -54,6 +54,9 @@ __device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b)
     asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
     return d;
 }
+
+// a pixel of zeros (loaded like any other: cleared in a branch, the registers cost a select each)
+__device__ const float2 __align__(16) g_zero[4] = {};
 
 // The per-entry reduction buffers 64 / (2P) entries of 2P lane partials: slot b holds lane l's
 // component c at b * (33 * 2P) + l * 2P + c (one 2P-float pad per slot, so that the 32 lanes'
@@ -93,47 +96,29 @@ __device__ __forceinline__ int degrid_entries(Chunk<P, false>& ck, int j, int S,
     };
     unsigned toff[NU];
     place_classes<NU, PB>(toff, ck.cls, ck.cur, ck.e[j], S, un.x, un.y, lane);
-    // The pairs' pixels.  P = 1: the two points' real parts and imaginary parts as packed pairs, as the
-    // samples come.  P = 2, 4: per point, two polarisations' parts as packed pairs, multiplied by a sample's part as
-    // a scalar (FMAs that read five registers run at 2.6 cycles against 3.2 for three pairs, and the
-    // sums need no addition across a pair: 1650 -> 1600 us on 0.87 M entries of supports 9..65).
-    constexpr int Q = P == 1 ? 1 : P / 2;      // pairs of polarisations
-    f32x2 g[NU][2][Q][2];                      // P = 1: [u][0][0] = {re, re'}, {im, im'}; else [u][point][q] = re, im
+    // The pairs' pixels, each polarisation (re, im) in the registers that the loads fill: a layout that took moves
+    // (the two points', or two polarisations', parts side by side) waited for each pair's loads before the next pair's
+    // were issued (3 M entries of support 15 at P = 4, each two columns and a row from the one before: 3.36 -> 2.50 ms).
+    f32x2 g[NU][2][P];
 #pragma unroll
     for (int u = 0; u < NU; ++u)
 #pragma unroll
-        for (int h = 0; h < 2; ++h)
+        for (int p = 0; p < P; ++p) g[u][0][p] = g[u][1][p] = 0ull;
+    // What a move of the footprint does to the pairs' pixels, a bit a unit at: kA and kB the first or the second row's
+    // pixel is loaded; kZ the second row is the one past the footprint: 0 is loaded (its samples are 0, what lies
+    // there may be an infinity).
+    constexpr int kA = 0, kB = NU, kZ = 2 * NU;
+    const float2* gch = grid + (size_t)ch * tp.N * tp.N * P;
+    auto reload = [&](unsigned todo) {
+        int cur[NU];
 #pragma unroll
-            for (int q = 0; q < Q; ++q) g[u][h][q][0] = g[u][h][q][1] = 0ull;
-    // loads the pairs in `which` for the footprint whose first row is y0; the row past the footprint stays
-    // 0 (its samples are 0, its pixels may hold an infinity)
-    auto reload = [&](unsigned which, int y0) {
+        for (int u = 0; u < NU; ++u) cur[u] = ck.cur[u][lane];
 #pragma unroll
         for (int u = 0; u < NU; ++u) {
-            if (which & (1u << u)) {
-                const int cur = ck.cur[u][lane];
-                if (cur >= 0) {
-                    const int y = cur >> 16;
-                    const float2* px = grid + ((size_t)((unsigned)ch * (unsigned)tp.N + (unsigned)y) * tp.N + (cur & 0xFFFF)) * P;
-                    float2 a[P], b[P];
-                    load_pixel<P>(px, a);
-#pragma unroll
-                    for (int p = 0; p < P; ++p) b[p] = make_float2(0.f, 0.f);
-                    if (y + H < y0 + S) load_pixel<P>(px + (size_t)(H * tp.N) * P, b);
-                    if constexpr (P == 1) {
-                        g[u][0][0][0] = pack2(a[0].x, b[0].x);
-                        g[u][0][0][1] = pack2(a[0].y, b[0].y);
-                    } else {
-#pragma unroll
-                        for (int q = 0; q < Q; ++q) {
-                            g[u][0][q][0] = pack2(a[2 * q].x, a[2 * q + 1].x);
-                            g[u][0][q][1] = pack2(a[2 * q].y, a[2 * q + 1].y);
-                            g[u][1][q][0] = pack2(b[2 * q].x, b[2 * q + 1].x);
-                            g[u][1][q][1] = pack2(b[2 * q].y, b[2 * q + 1].y);
-                        }
-                    }
-                }
-            }
+            const float2* a = gch + (size_t)linear(cur[u], tp.N, 1u) * P;
+            const float2* b = todo & (1u << (kZ + u)) ? g_zero : a + (size_t)(H * tp.N) * P;
+            if (todo & (1u << (kA + u))) load_pixel<P>(a, g[u][0]);
+            if (todo & (1u << (kB + u))) load_pixel<P>(b, g[u][1]);
         }
     };
     KPair k[NU];
@@ -143,54 +128,35 @@ __device__ __forceinline__ int degrid_entries(Chunk<P, false>& ck, int j, int S,
         for (int u = 0; u < NU; ++u) k[u] = load_pair((const float2*)nullptr, kz, toff[u]);
     }
     // an entry's sums into the reduction buffer; the samples of the entry whose sub-kernel is at kz are loaded
-    // into a unit's registers behind its FMAs
-    auto entry = [&](const char* kz) {
-        // conj(k) g = (kx gx + ky gy, kx gy - ky gx)
+    // into a unit's registers behind its FMAs, and then() loads pixels (at P = 4 only once the sums have left the
+    // registers: 2091 -> 1788 us on those 3 M entries, with 4 bytes of spills for 24)
+    auto entry = [&](const char* kz, auto then) {
+        // conj(k) g = (kx gx + ky gy, kx gy - ky gx), from the sums of kx (gx, gy) and ky (gx, gy)
         float v[V];
-        if constexpr (P == 1) {
-            f32x2 s0 = 0ull, s1 = 0ull;
+        f32x2 sx[P], sy[P];
 #pragma unroll
-            for (int u = 0; u < NU; ++u) {
-                const float2 im = unpack2(k[u].im);
-                s0 = fma2(k[u].im, g[u][0][0][1], fma2(k[u].re, g[u][0][0][0], s0));
-                s1 = fma2(pack2(-im.x, -im.y), g[u][0][0][0], fma2(k[u].re, g[u][0][0][1], s1));
-                k[u] = load_pair((const float2*)nullptr, kz, toff[u]);
-            }
-            const float2 a = unpack2(s0), b = unpack2(s1);
-            v[0] = a.x + a.y;
-            v[1] = b.x + b.y;
-        } else {
-            f32x2 s[Q][2];
+        for (int p = 0; p < P; ++p) sx[p] = sy[p] = 0ull;
 #pragma unroll
-            for (int q = 0; q < Q; ++q) s[q][0] = s[q][1] = 0ull;
+        for (int u = 0; u < NU; ++u) {
+            const float2 re = unpack2(k[u].re), im = unpack2(k[u].im);
 #pragma unroll
-            for (int u = 0; u < NU; ++u) {
-                const float2 re = unpack2(k[u].re), im = unpack2(k[u].im);
+            for (int h = 0; h < 2; ++h) {
+                const float x = h ? re.y : re.x, y = h ? im.y : im.x;
+                const f32x2 kx = pack2(x, x), ky = pack2(y, y);
 #pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const float x = h ? re.y : re.x, y = h ? im.y : im.x;
-                    const f32x2 kx = pack2(x, x), ky = pack2(y, y), ny = pack2(-y, -y);
-#pragma unroll
-                    for (int q = 0; q < Q; ++q) {
-                        s[q][0] = fma2(kx, g[u][h][q][0], s[q][0]);
-                        s[q][1] = fma2(kx, g[u][h][q][1], s[q][1]);
-                    }
-#pragma unroll
-                    for (int q = 0; q < Q; ++q) {
-                        s[q][0] = fma2(ky, g[u][h][q][1], s[q][0]);
-                        s[q][1] = fma2(ny, g[u][h][q][0], s[q][1]);
-                    }
+                for (int p = 0; p < P; ++p) {
+                    sx[p] = fma2(kx, g[u][h][p], sx[p]);
+                    sy[p] = fma2(ky, g[u][h][p], sy[p]);
                 }
-                k[u] = load_pair((const float2*)nullptr, kz, toff[u]);
             }
+            k[u] = load_pair((const float2*)nullptr, kz, toff[u]);
+        }
+        if constexpr (P < 4) then();
 #pragma unroll
-            for (int q = 0; q < Q; ++q) {
-                const float2 a = unpack2(s[q][0]), b = unpack2(s[q][1]);
-                v[4 * q] = a.x;
-                v[4 * q + 1] = b.x;
-                v[4 * q + 2] = a.y;
-                v[4 * q + 3] = b.y;
-            }
+        for (int p = 0; p < P; ++p) {
+            const float2 a = unpack2(sx[p]), b = unpack2(sy[p]);
+            v[2 * p] = a.x + b.y;
+            v[2 * p + 1] = a.y - b.x;
         }
         float* dst = red + nbuf * SLOT + lane * V;
         if constexpr (V == 8) {
@@ -205,9 +171,20 @@ __device__ __forceinline__ int degrid_entries(Chunk<P, false>& ck, int j, int S,
             *reinterpret_cast<float2*>(dst) = make_float2(v[0], v[1]);
         }
         ++nbuf;
+        if constexpr (P == 4) then();
     };
-    unsigned touched = ~0u;           // pairs whose pixels change with the coming entry
-    int y0 = ck.e[j].x >> 16;
+    const unsigned minus_sh = minus_moduli(S, H);
+    // the first pixel (column | row << 16) of a pair whose second row is the one past the footprint: at least this
+    int edge = ((ck.e[j].x >> 16) + H - 1) << 16;
+    {
+        unsigned todo = 0;
+#pragma unroll
+        for (int u = 0; u < NU; ++u) {
+            const int cur = ck.cur[u][lane];
+            if (cur >= 0) todo |= (1u << (kA + u)) | (cur < edge ? 1u << (kB + u) : 0u);
+        }
+        reload(todo);
+    }
     bool same = true;
     for (;;) {
         if (nbuf == NB || !same) {
@@ -216,17 +193,13 @@ __device__ __forceinline__ int degrid_entries(Chunk<P, false>& ck, int j, int S,
             nbuf = 0;
             if (!same) return j;
         }
-        if (touched) {
-            reload(touched, y0);
-            touched = 0;
-        }
         // entries whose successor has the same footprint, as far as the buffer goes
         const unsigned later = ck.mv & (0xFFFFFFFEu << j);
         const int last = (later ? __ffs(later) - 1 : ck.cnt) - 1, stop = min(last, j + NB - nbuf);
-        for (; j < stop; ++j) entry(table + (size_t)ck.z[j + 1] * PB);
+        for (; j < stop; ++j) entry(table + (size_t)ck.z[j + 1] * PB, [] {});
         if (nbuf == NB) continue;
-        // the footprint's last entry in the chunk: the move to its successor comes first (as in the gridder)
-        unsigned zn = ck.z[j];
+        // the footprint's last entry in the chunk: its successor's sample offsets come first (as in the gridder)
+        unsigned zn = ck.z[j], todo = 0;
         bool more = true;
         if (++j == ck.cnt) {
             more = ck.next(tp, report);
@@ -236,43 +209,29 @@ __device__ __forceinline__ int degrid_entries(Chunk<P, false>& ck, int j, int S,
         if (same) {
             zn = ck.z[j];
             if ((ck.mv >> j) & 1) {
-                const Move m = ck.m[j];
-                if (m.w == -1) {
-                    // a jump: the pairs whose pixels change are loaded, and on another row those whose second row is
-                    // or was the one past the footprint.  (As the start of a run it drained the sums and loaded every
-                    // pixel: steps of 10 s on a 4000^2 grid, 2.24 -> 2.14 ms at P = 4, 1.63 -> 1.54 at P = 2.)
-                    const Staged E = ck.e[j];
-                    const int y1 = E.x >> 16;
+                // Every pair is placed anew, and of its two pixels those loaded that it does not hold (on lists that move
+                // by one column now and then, a path of its own for that move gained nothing: 1523 against 1505 us).
+                const Staged E = ck.e[j];
+                const int edge1 = ((E.x >> 16) + H - 1) << 16;
 #pragma unroll
-                    for (int u = 0; u < NU; ++u) {
-                        const int2 d = place_class(ck.cls[u][lane], E, S, H);
-                        const int cur = ck.cur[u][lane], n = E.x + (d.x | (d.y << 16));
-                        toff[u] = (unsigned)(d.y * S + d.x) * PB;
-                        if (cur >= 0 && (n != cur || (y1 != y0 && (d.y == H - 1 || (cur >> 16) - y0 == H - 1)))) {
-                            ck.cur[u][lane] = n;
-                            touched |= 1u << u;
-                        }
-                    }
-                    y0 = y1;
-                } else {
-                    touched = move_classes<NU, PB>(toff, ck.cls, m, lane);
-                    y0 = ck.e[j].x >> 16;
-                    const bool row = (m.w >> 16) != 0x4410;
-                    const int c = m.w & 0xFFFF, before = c ? c - 1 : H - 1;
-#pragma unroll
-                    for (int u = 0; u < NU; ++u) {
-                        if (touched & (1u << u)) {
-                            const int cur = ck.cur[u][lane];
-                            if (cur >= 0) ck.cur[u][lane] = cur + m.z;
-                        }
-                        // a row move also brings the class row before the one that wraps next to the row past the
-                        // footprint, or away from it
-                        if (row && (ck.cls[u][lane] >> 16) == before) touched |= 1u << u;
+                for (int u = 0; u < NU; ++u) {
+                    const int d = place_class(ck.cls[u][lane], E, minus_sh);
+                    const int cur = ck.cur[u][lane], n = E.x + d;
+                    toff[u] = linear(d, S, PB);
+                    if (cur >= 0) {
+                        const bool moved = n != cur, past = n >= edge1;
+                        ck.cur[u][lane] = n;
+                        todo |= (moved ? 1u << (kA + u) : 0u) | (moved || past != (cur >= edge) ? 1u << (kB + u) : 0u) |
+                                (past ? 1u << (kZ + u) : 0u);
                     }
                 }
+                edge = edge1;
             }
         }
-        entry(table + (size_t)zn * PB);
+        // the pixels are on their way before the sums are drained
+        entry(table + (size_t)zn * PB, [&] {
+            if (todo) reload(todo);
+        });
     }
 }
 

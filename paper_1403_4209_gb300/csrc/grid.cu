@@ -287,6 +287,7 @@ __device__ __forceinline__ int jump_entries(Chunk<P, true>& ck, int j, int unit0
     const int key = e[j].w, S = key_support(key), ch = key_chan(key), H = (S + 1) >> 1;
     const float inv_s = 1.0f / (float)S;
     const int end = min(H * S, unit1 * 32);
+    const unsigned minus_sh = minus_moduli(S, H);
     int cls[NU], cur[NU];                        // as place_classes' (a lane past the last pair: cur = -1)
     f32x2 acc[NU][P][2];
     KPair k[NU];
@@ -298,9 +299,9 @@ __device__ __forceinline__ int jump_entries(Chunk<P, true>& ck, int j, int unit0
             const int i = (unit0 + u) * 32 + lane;
             const int2 vu = divmod_small(i < end ? i : 0, S, inv_s);
             cls[u] = vu.y | (vu.x << 16);
-            const int2 d = place_class(cls[u], E, S, H);
-            cur[u] = i < end ? E.x + (d.x | (d.y << 16)) : -1;
-            k[u] = load_pair((const TS*)nullptr, kz, (unsigned)(d.y * S + d.x) * PB);
+            const int d = place_class(cls[u], E, minus_sh);
+            cur[u] = i < end ? E.x + d : -1;
+            k[u] = load_pair((const TS*)nullptr, kz, linear(d, S, PB));
 #pragma unroll
             for (int p = 0; p < P; ++p) acc[u][p][0] = acc[u][p][1] = 0ull;
         }
@@ -326,9 +327,9 @@ __device__ __forceinline__ int jump_entries(Chunk<P, true>& ck, int j, int unit0
                 acc[u][p][0] = fma2(ny, k[u].im, fma2(gx, k[u].re, acc[u][p][0]));
                 acc[u][p][1] = fma2(gx, k[u].im, fma2(gy, k[u].re, acc[u][p][1]));
             }
-            const int2 d = place_class(cls[u], E, S, H);
-            if (more) k[u] = load_pair((const TS*)nullptr, kz, (unsigned)(d.y * S + d.x) * PB);
-            const int next = E.x + (d.x | (d.y << 16));
+            const int d = place_class(cls[u], E, minus_sh);
+            if (more) k[u] = load_pair((const TS*)nullptr, kz, linear(d, S, PB));
+            const int next = E.x + d;
             if (cur[u] >= 0 && (!more || next != cur[u])) {
                 if constexpr (P == 4) {
                     // one row of the pair may stay in the footprint, as the other row of the pair now held

@@ -126,7 +126,7 @@ typedef int4 Staged;
 // A move of the footprint by one column or row: every pair's sample offset (in pairs) shifts by x; the
 // one class column (or row) that left the footprint wraps to the other side, its offset shifts by y;
 // z: what is added to a wrapped pair's first pixel (column | row << 16);
-// w: the class | the byte selector of its axis in a packed class << 16; -1 (the degridder's): a jump.
+// w: the class | the byte selector of its axis in a packed class << 16.
 typedef int4 Move;
 __device__ __forceinline__ int key_support(int key) { return key >> 16; }
 __device__ __forceinline__ int key_chan(int key) { return key & 0xFFFF; }
@@ -194,13 +194,20 @@ __device__ __forceinline__ unsigned move_classes(unsigned (&toff)[NU], const int
     return wraps;
 }
 
-// Places a pair of class cl (column | row << 16) in the footprint of entry E: its column and row there.
-__device__ __forceinline__ int2 place_class(int cl, const Staged& E, int S, int H)
+// Places a pair of class cl (column | row << 16) in the footprint of entry E: its column | row << 16 there.  Each
+// half of cl + E.y is less than twice its modulus, so that the smaller of it and it less the modulus (as an unsigned
+// 16-bit number) is the remainder; minus_sh = minus_moduli(S, H).
+__device__ __forceinline__ unsigned minus_moduli(int S, int H) { return (unsigned)(0x10000 - S) | ((unsigned)(0x10000 - H) << 16); }
+__device__ __forceinline__ int place_class(int cl, const Staged& E, unsigned minus_sh)
 {
-    int du = (cl & 0xFFFF) + (E.y & 0xFFFF), dv = (cl >> 16) + (E.y >> 16);
-    du -= (du >= S) ? S : 0;
-    dv -= (dv >= H) ? H : 0;
-    return make_int2(du, dv);
+    const unsigned t = (unsigned)cl + (unsigned)E.y;
+    return (int)__viaddmin_u16x2(t, minus_sh, t);
+}
+
+// column + row * pitch of a packed column | row << 16 (modulo 2^32), times scale
+__device__ __forceinline__ unsigned linear(int packed, int pitch, unsigned scale)
+{
+    return (unsigned)packed * scale + (unsigned)(packed >> 16) * ((unsigned)(pitch - 0x10000) * scale);
 }
 
 constexpr int kPartMin = 4;   // entries of the shortest part of a segment
@@ -223,10 +230,11 @@ __device__ __forceinline__ int2 block_units(int S, int blk, int nb)
 template <int P, bool GAMMA>
 struct Chunk {
     static constexpr int kG = GAMMA ? 32 * P * (int)sizeof(float2) : 0;
-    static constexpr int kBytes = 3 * 32 * (int)sizeof(int4) + 2 * kG + (2 * kUnitsMax + 1) * 32 * (int)sizeof(int);
+    static constexpr int kM = GAMMA ? 32 : 0;
+    static constexpr int kBytes = (64 + kM) * (int)sizeof(int4) + 2 * kG + (2 * kUnitsMax + 1) * 32 * (int)sizeof(int);
     int4* raw_e;             // [32] as copied
     Staged* e;               // [32]
-    Move* m;                 // [32] from the entry's predecessor (entries of mv that are not of kc)
+    Move* m;                 // [32] from the entry's predecessor (entries of mv that are not of kc; the gridder's)
     float2* raw_g;           // [32][P]
     float2* g;               // [32][P] weighted visibilities
     unsigned* z;             // [32] the entries' z again
@@ -240,7 +248,7 @@ struct Chunk {
     unsigned slow;           // entries with an infinite or NaN visibility
 
     __device__ __forceinline__ Chunk(unsigned char* base, int lane_)
-        : raw_e(reinterpret_cast<int4*>(base)), e(raw_e + 32), m(e + 32), raw_g(reinterpret_cast<float2*>(m + 32)),
+        : raw_e(reinterpret_cast<int4*>(base)), e(raw_e + 32), m(e + 32), raw_g(reinterpret_cast<float2*>(m + kM)),
           g(raw_g + kG / sizeof(float2)), z(reinterpret_cast<unsigned*>(g + kG / sizeof(float2))),
           cls(reinterpret_cast<int (*)[32]>(z + 32)), cur(cls + kUnitsMax), lane(lane_)
     {
@@ -312,21 +320,23 @@ struct Chunk {
             qk = pkey;
             qf = last.x;
         }
-        // the move from the predecessor
-        const int S = key_support(s.w), H = (S + 1) >> 1;
-        const int dx = (s.x & 0xFFFF) - (qf & 0xFFFF), dy = (s.x >> 16) - (qf >> 16);
-        const bool along_x = dy == 0;
-        const int d = dx + dy, md = along_x ? S : H, step = along_x ? 1 : S;
-        const int cn = along_x ? s.y & 0xFFFF : s.y >> 16;                 // (-origin) mod md
-        const int o = cn ? md - cn : 0;                                    // origin mod md
-        const int c = d > 0 ? (o ? o - 1 : md - 1) : o;                    // the class that wraps
-        const bool far = abs(dx) + abs(dy) > 1;
-        const bool k = s.w != qk || sl || qs || (GAMMA && far);
+        bool k = s.w != qk || sl || qs;
+        if constexpr (GAMMA) {
+            // the move from the predecessor
+            const int S = key_support(s.w), H = (S + 1) >> 1;
+            const int dx = (s.x & 0xFFFF) - (qf & 0xFFFF), dy = (s.x >> 16) - (qf >> 16);
+            const bool along_x = dy == 0;
+            const int d = dx + dy, md = along_x ? S : H, step = along_x ? 1 : S;
+            const int cn = along_x ? s.y & 0xFFFF : s.y >> 16;             // (-origin) mod md
+            const int o = cn ? md - cn : 0;                                // origin mod md
+            const int c = d > 0 ? (o ? o - 1 : md - 1) : o;                // the class that wraps
+            k = k || abs(dx) + abs(dy) > 1;
+            m[lane] = make_int4(-d * step, d * (md - 1) * step, along_x ? d * S : d * H * 65536,
+                                c | ((along_x ? 0x4410 : 0x4432) << 16));
+        }
         kc = __ballot_sync(0xffffffffu, in && k);
         mv = __ballot_sync(0xffffffffu, in && (k || s.x != qf));
         e[lane] = s;
-        m[lane] = make_int4(-d * step, d * (md - 1) * step, along_x ? d * S : d * H * 65536,
-                            !GAMMA && far ? -1 : c | ((along_x ? 0x4410 : 0x4432) << 16));
         z[lane] = (unsigned)s.z;
         if constexpr (GAMMA) {
 #pragma unroll
