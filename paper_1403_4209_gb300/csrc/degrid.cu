@@ -83,14 +83,15 @@ __device__ __forceinline__ int degrid_entries(Chunk<P, false>& ck, int j, int S,
         const int b = (2 * lane) / V, c = (2 * lane) % V;
         if (b < n) {
             const float* src = red + b * SLOT + c;
-            f32x2 t = 0ull;
+            f32x2 t[4] = {0ull, 0ull, 0ull, 0ull};      // four chains: shorter, and a quarter of the rounding steps each
 #pragma unroll
             for (int l2 = 0; l2 < 32; ++l2) {
                 // V = 8: lanes with bit 2 set stored their two 16-byte halves swapped
                 const int cs = (V == 8 && (l2 & 4)) ? 4 : 0;
-                t = add2(t, *reinterpret_cast<const f32x2*>(src + l2 * V + (c ^ cs) - c));
+                t[l2 & 3] = add2(t[l2 & 3], *reinterpret_cast<const f32x2*>(src + l2 * V + (c ^ cs) - c));
             }
-            atomicAdd(reinterpret_cast<float2*>(acc + (size_t)(eb + b) * V + c), unpack2(t));
+            atomicAdd(reinterpret_cast<float2*>(acc + (size_t)(eb + b) * V + c),
+                      unpack2(add2(add2(t[0], t[1]), add2(t[2], t[3]))));
         }
         __syncwarp();
     };
