@@ -270,7 +270,7 @@ int worklist_destroy(wg_worklist* h)
 {
     if (!h) return WG_OK;
     WorkList& w = h->w;
-    void* ptrs[] = {w.rinfo, w.rclass, w.tile_cnt, w.carry_q, w.carry_last, w.entries, w.gamma, w.runs, w.dacc, w.seg_nblk, w.seg_off, w.seg_offj,
+    void* ptrs[] = {w.rinfo, w.rclass, w.tile_cnt, w.carry_q, w.carry_last, w.entries, w.gamma, w.runs, w.dacc, w.seg_nblk, w.seg_off,
                     w.scal, w.chan_base, w.norm_priv, w.norm_batch, w.stat_priv, w.stats, w.stats_batch, w.task_counter};
     for (void* p : ptrs) cudaFree(p);
     delete h;
@@ -320,7 +320,6 @@ static int create_worklist(int64_t max_records, int64_t max_entries, int32_t C, 
     if (dacc) al((void**)&w.dacc, sizeof(float2) * max_entries * P);
     al((void**)&w.seg_nblk, sizeof(int) * w.seg_cap);
     al((void**)&w.seg_off, sizeof(int) * (w.seg_cap + 1));
-    al((void**)&w.seg_offj, sizeof(int) * (w.seg_cap + 1));
     al((void**)&w.scal, sizeof(long long) * 8);
     al((void**)&w.chan_base, sizeof(int) * (C + 1));
     al((void**)&w.norm_priv, sizeof(double) * kNormSlots * C * P);

@@ -391,7 +391,7 @@ static int degrid_sum_launch(const Grid& g, const Table& t, const WorkList& wl, 
             blocks_per_sm = 1;
     }
     k_degrid_sum<P><<<num_sms() * blocks_per_sm, kWarps * 32, smem, s>>>(
-        task_params(g, t, wl, wl.task_counter + 1, false), reinterpret_cast<const char*>(t.pairs), g.data,
+        task_params(g, t, wl, wl.task_counter + 1), reinterpret_cast<const char*>(t.pairs), g.data,
         reinterpret_cast<float*>(wl.dacc));
     WG_LAUNCHED("k_degrid_sum");
     return WG_OK;

@@ -6,7 +6,6 @@
 // kUnitsMax point pairs of the footprint by their class (pairs.cuh), so lanes never touch the same
 // pixel and accumulate in registers while the pair stays the same; when it moves, the lane flushes
 // its accumulators with vector FP32 atomics (all polarisations of a pixel are contiguous).
-// Segments whose footprints mostly jump are left to k_grid_jumps.
 //
 // What bounds it: instruction issue and the FMA pipe (59 % and 50 % busy at four polarisations, 128
 // registers, 16 warps an SM), then the L1 data path (68 %: every sample is used once per entry and comes from L2).
@@ -93,9 +92,13 @@ __device__ __forceinline__ void flush_pair(float2* __restrict__ grid, float2* __
     if (y + H < N) flush_pixel<P, COMP>(grid, errgrid, pix + (size_t)(H * N), b);
 }
 
-// One run of entries from entry j of the chunk on (same support and channel, the footprint moving by
-// at most one column or row at a time): the units [un.x, un.y) of the footprint, at most NU.  Returns
-// the first entry (of the chunk then staged) after it, or -1 at the item's end.  The code is kept
+// One run of entries from entry j of the chunk on (same support and channel): the units [un.x, un.y) of the
+// footprint, at most NU.  Returns the first entry (of the chunk then staged) after it, or -1 at the item's
+// end.  However the footprint moves, its pairs are placed anew and only those whose pixels change are flushed: runs that
+// ended at a jump flushed the whole footprint, which took longer than single points did, and added more
+// rounding steps (4.8 M records of 10 s steps on 4000^2, P = 4, 256 entries: 7.27 -> 5.95 ms; single points 7.26).
+// A pair that moves by H rows keeps one of its pixels in the other place; to keep its sum as well cost more
+// instructions than its flush (1225 -> 1352 us on 4.8 M records, P = 4).  The code is kept
 // small, with one copy of the staging, the move and the flush: a kernel with several of each and
 // variants for more values of NU stalled on instruction fetch half of its time.
 template <int P, typename TS, bool COMP, int NU>
@@ -137,14 +140,16 @@ __device__ __forceinline__ int run_entries(Chunk<P, true>& ck, int j, int S, int
         // entries whose successor has the same footprint
         const unsigned later = ck.mv & (0xFFFFFFFEu << j);
         const int last = (later ? __ffs(later) - 1 : ck.cnt) - 1;
+        // (unrolled, the loop holds more values than there are registers at P = 4: 22.2 against 20.5 ms on 116 M records)
+#pragma unroll(P == 4 ? 1 : 2)
         for (; j < last; ++j) {
             float2 g[P];
 #pragma unroll
             for (int p = 0; p < P; ++p) g[p] = ck.g[j * P + p];
             add(g, table + (size_t)ck.z[j + 1] * PB);
         }
-        // the footprint's last entry in the chunk: its successor's offsets are moved first, so that its samples
-        // can be loaded behind the FMAs; the pairs that wrap are flushed after them
+        // the footprint's last entry in the chunk: the pairs are placed in its successor's footprint first, so that its samples
+        // can be loaded behind the FMAs; those that move are flushed after them
         float2 g[P];
 #pragma unroll
         for (int p = 0; p < P; ++p) g[p] = ck.g[j * P + p];
@@ -155,25 +160,30 @@ __device__ __forceinline__ int run_entries(Chunk<P, true>& ck, int j, int S, int
             j = more ? 0 : -1;
         }
         const bool same = more && !((ck.kc >> j) & 1);       // the run goes on
-        unsigned wraps = ~0u;
-        int step = 0;
+        unsigned moves = ~0u;                                // units whose pairs move
         if (same) {
             zn = ck.z[j];
-            wraps = 0;
+            moves = 0;
             if ((ck.mv >> j) & 1) {
-                const Move m = ck.m[j];
-                wraps = move_classes<NU, PB>(toff, ck.cls, m, lane);
-                step = m.z;
+                const Staged E = ck.e[j];
+                const unsigned minus_sh = minus_moduli(S, H);
+#pragma unroll
+                for (int u = 0; u < NU; ++u) {
+                    const int d = place_class(ck.cls[u][lane], E, minus_sh), n = E.x + d;
+                    toff[u] = linear(d, S, PB);
+                    ck.nxt[u][lane] = n;
+                    moves |= n != ck.cur[u][lane] ? 1u << u : 0u;
+                }
             }
         }
         add(g, table + (size_t)zn * PB);
 #pragma unroll
         for (int u = 0; u < NU; ++u) {
-            if (wraps & (1u << u)) {
+            if (moves & (1u << u)) {
                 const int cur = ck.cur[u][lane];
                 if (cur >= 0) {
                     flush_pair<P, COMP>(grid, errgrid, ch, cur, H, tp.N, acc[u]);
-                    ck.cur[u][lane] = cur + step;
+                    ck.cur[u][lane] = ck.nxt[u][lane];
                 }
             }
         }
@@ -209,6 +219,22 @@ __device__ __noinline__ void slow_entry(const float2* g, int S, int unit0, int u
 
 }  // namespace
 
+// adds the batch normaliser and statistics into the grid's accumulators; the batch's normaliser
+// row c goes to grid channel c * stride (w-stacking keeps a channel's N_p in its plane 0)
+struct AccumulateParams {
+    double* gnorm;
+    const double* bnorm;
+    int n, P, stride;
+    unsigned long long* gcnt;
+    const unsigned long long* bcnt;
+};
+__device__ __forceinline__ void accumulate(const AccumulateParams& a, int i)
+{
+    if (i < a.n) a.gnorm[(size_t)(i / a.P) * a.stride * a.P + i % a.P] += a.bnorm[i];
+    if (i < ST_N) a.gcnt[i] += a.bcnt[i];
+}
+__global__ void k_accumulate(AccumulateParams a) { accumulate(a, threadIdx.x + blockIdx.x * blockDim.x); }
+
 // SMALL: every support of the table has at most kSmallPairs pairs, two units (up to support 9).  Two units a lane leave
 // registers for five blocks an SM, and none idle: support 7 at P = 4 from 387 to 226 us, support 9 from 409 to 241,
 // compensated from 713 to 551 (single points took 281, 332 and 666).
@@ -217,16 +243,20 @@ template <int P, typename TS, bool COMP, bool SMALL>
 __global__ void __launch_bounds__(kWarps * 32, P == 4 ? (SMALL ? 5 : 4) : P == 2 ? 5 : 7) k_grid(TaskParams tp,
                                                                                                 const char* __restrict__ table,
                                                                                                 float2* __restrict__ grid,
-                                                                                                float2* __restrict__ errgrid)
+                                                                                                float2* __restrict__ errgrid,
+                                                                                                AccumulateParams acc)
 {
     __shared__ __align__(16) unsigned char smem[kWarps * Chunk<P, true>::kBytes];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    if (acc.gnorm) {
+        const int m = max(acc.n, (int)ST_N);
+        for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < m; i += gridDim.x * blockDim.x) accumulate(acc, i);
+    }
     Chunk<P, true> ck(smem + wid * Chunk<P, true>::kBytes, lane);
     const int parts = item_parts(tp);
 
     Item it;
     while (next_item(tp, parts, lane, it)) {
-        if (__ldg(&tp.seg_nblk[it.seg]) & kSegJumps) continue;      // k_grid_jumps takes it
         // an item whose share of some support is more than kUnitsMax units takes the rest in a second pass
         bool again = it.n > 0;
         for (int pass = 0; again; ++pass) {
@@ -252,11 +282,13 @@ __global__ void __launch_bounds__(kWarps * 32, P == 4 ? (SMALL ? 5 : 4) : P == 2
                     j = ck.run_end(j);
                     continue;
                 }
+                const size_t plane = (size_t)ch * tp.N * tp.N * P;
+                float2* gch = grid + plane;
+                float2* ech = COMP ? errgrid + plane : nullptr;
                 if ((ck.slow >> j) & 1) {
                     const Staged e = ck.e[j];
                     slow_entry<P, TS, COMP>(ck.g + j * P, S, un.x, un.y, e.x,
-                                            table + (size_t)(unsigned)e.z * kPairBytes<TS>, tp.N, lane,
-                                            grid + (size_t)ch * tp.N * tp.N * P, COMP ? errgrid + (size_t)ch * tp.N * tp.N * P : nullptr);
+                                            table + (size_t)(unsigned)e.z * kPairBytes<TS>, tp.N, lane, gch, ech);
                     ++j;
                     continue;
                 }
@@ -267,172 +299,6 @@ __global__ void __launch_bounds__(kWarps * 32, P == 4 ? (SMALL ? 5 : 4) : P == 2
                     j = run_entries<P, TS, COMP, kUnitsMax>(ck, j, S, ch, un, tp, report, table, grid, errgrid);
                 else
                     j = run_entries<P, TS, COMP, 2>(ck, j, S, ch, un, tp, report, table, grid, errgrid);
-            }
-        }
-    }
-}
-
-// Entries from j on whose footprints jump about: the units [unit0, unit1) of a footprint, at most kUnitsMax, up to a
-// slow entry, or another support or channel.  Each entry is placed anew, and only
-// the pairs whose pixels change are flushed (a jump of two columns and a row leaves most of a footprint where it was).
-// Returns the first entry (of the chunk then staged) not taken, or -1 at the item's end.
-template <int P, typename TS, bool COMP>
-__device__ __forceinline__ int jump_entries(Chunk<P, true>& ck, int j, int unit0, int unit1, const TaskParams& tp, bool report,
-                                            const char* __restrict__ table, float2* __restrict__ grid,
-                                            float2* __restrict__ errgrid)
-{
-    constexpr int PB = kPairBytes<TS>, NU = kUnitsMax;
-    const int lane = ck.lane, N = tp.N;
-    const Staged* e = ck.e;
-    const int key = e[j].w, S = key_support(key), ch = key_chan(key), H = (S + 1) >> 1;
-    const float inv_s = 1.0f / (float)S;
-    const int end = min(H * S, unit1 * 32);
-    const unsigned minus_sh = minus_moduli(S, H);
-    int cls[NU], cur[NU];                        // as place_classes' (a lane past the last pair: cur = -1)
-    f32x2 acc[NU][P][2];
-    KPair k[NU];
-    {
-        const Staged E = e[j];
-        const char* kz = table + (size_t)(unsigned)E.z * PB;
-#pragma unroll
-        for (int u = 0; u < NU; ++u) {
-            const int i = (unit0 + u) * 32 + lane;
-            const int2 vu = divmod_small(i < end ? i : 0, S, inv_s);
-            cls[u] = vu.y | (vu.x << 16);
-            const int d = place_class(cls[u], E, minus_sh);
-            cur[u] = i < end ? E.x + d : -1;
-            k[u] = load_pair((const TS*)nullptr, kz, linear(d, S, PB));
-#pragma unroll
-            for (int p = 0; p < P; ++p) acc[u][p][0] = acc[u][p][1] = 0ull;
-        }
-    }
-    for (;;) {
-        float2 g[P];
-#pragma unroll
-        for (int p = 0; p < P; ++p) g[p] = ck.g[j * P + p];
-        bool more = true;
-        if (++j == ck.cnt) {
-            more = ck.next(tp, report);
-            j = more ? 0 : -1;
-        }
-        more = more && !((ck.slow >> j) & 1) && e[j].w == key;
-        const Staged E = e[max(j, 0)];
-        const char* kz = table + (size_t)(unsigned)E.z * PB;
-#pragma unroll
-        for (int u = 0; u < NU; ++u) {
-            if (unit0 + u >= unit1) break;
-#pragma unroll
-            for (int p = 0; p < P; ++p) {
-                const f32x2 gx = pack2(g[p].x, g[p].x), gy = pack2(g[p].y, g[p].y), ny = pack2(-g[p].y, -g[p].y);
-                acc[u][p][0] = fma2(ny, k[u].im, fma2(gx, k[u].re, acc[u][p][0]));
-                acc[u][p][1] = fma2(gx, k[u].im, fma2(gy, k[u].re, acc[u][p][1]));
-            }
-            const int d = place_class(cls[u], E, minus_sh);
-            if (more) k[u] = load_pair((const TS*)nullptr, kz, linear(d, S, PB));
-            const int next = E.x + d;
-            if (cur[u] >= 0 && (!more || next != cur[u])) {
-                if constexpr (P == 4) {
-                    // one row of the pair may stay in the footprint, as the other row of the pair now held
-                    const bool low = more && next == cur[u] + (H << 16), high = more && next == cur[u] - (H << 16);
-                    const int y = cur[u] >> 16;
-                    const size_t pix = (size_t)((unsigned)ch * (unsigned)N + (unsigned)y) * N + (cur[u] & 0xFFFF);
-                    float2 a[P], b[P];
-#pragma unroll
-                    for (int p = 0; p < P; ++p) {
-                        const float2 re = unpack2(acc[u][p][0]), im = unpack2(acc[u][p][1]);
-                        a[p] = make_float2(re.x, im.x);
-                        b[p] = make_float2(re.y, im.y);
-                        acc[u][p][0] = pack2(low ? b[p].x : 0.f, high ? a[p].x : 0.f);
-                        acc[u][p][1] = pack2(low ? b[p].y : 0.f, high ? a[p].y : 0.f);
-                    }
-                    if (!high) flush_pixel<P, COMP>(grid, errgrid, pix, a);
-                    bool any = false;                // (the row past the footprint has only zeros)
-#pragma unroll
-                    for (int p = 0; p < P; ++p) any = any || b[p].x != 0.f || b[p].y != 0.f;
-                    if (any && !low && y + H < N) flush_pixel<P, COMP>(grid, errgrid, pix + (size_t)(H * N), b);
-                } else {
-                    flush_pair<P, COMP>(grid, errgrid, ch, cur[u], H, N, acc[u]);
-                }
-                cur[u] = next;
-            }
-        }
-        if (!more) return j;
-    }
-}
-
-// adds the batch normaliser and statistics into the grid's accumulators; the batch's normaliser
-// row c goes to grid channel c * stride (w-stacking keeps a channel's N_p in its plane 0)
-struct AccumulateParams {
-    double* gnorm;
-    const double* bnorm;
-    int n, P, stride;
-    unsigned long long* gcnt;
-    const unsigned long long* bcnt;
-};
-__device__ __forceinline__ void accumulate(const AccumulateParams& a, int i)
-{
-    if (i < a.n) a.gnorm[(size_t)(i / a.P) * a.stride * a.P + i % a.P] += a.bnorm[i];
-    if (i < ST_N) a.gcnt[i] += a.bcnt[i];
-}
-__global__ void k_accumulate(AccumulateParams a) { accumulate(a, threadIdx.x + blockIdx.x * blockDim.x); }
-
-// The segments whose footprints jump about (interleaved channels, long steps); k_segments marks them.  Run by run, as
-// k_grid takes a segment, an entry with a footprint of its own is placed, waits for its samples and is flushed whole:
-// 3.2 M entries of support 15, most a few cells from the one before, took 7.5 ms at P = 4 (twice the
-// vector reductions that are needed), here 2.9; support 7 at P = 2 1.39 against 0.63.  It is a kernel of its own because
-// at four polarisations it wants 160 registers (three blocks: 1.23 against 1.34 ms at support 7), and
-// because a call to it in k_grid's loop, taken or not, slowed that by 6 %.  Marked: segments with a jump in two entries
-// (P = 4: in six) or more; at P = 2 with jumps in one of four k_grid is faster (2.77 against 3.04 ms).
-// Bound by the reductions in L2 (54 % of its request rate) and their imbalance over its slices.
-// Also adds the batch's normaliser and statistics (acc.gnorm not null).
-template <int P, typename TS, bool COMP>
-__global__ void __launch_bounds__(kWarps * 32, P == 4 ? 3 : P == 2 ? 5 : 7) k_grid_jumps(TaskParams tp,
-                                                                                        const char* __restrict__ table,
-                                                                                        float2* __restrict__ grid,
-                                                                                        float2* __restrict__ errgrid,
-                                                                                        AccumulateParams acc)
-{
-    __shared__ __align__(16) unsigned char smem[kWarps * Chunk<P, true>::kBytes];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    if (acc.gnorm) {
-        const int m = max(acc.n, (int)ST_N);
-        for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < m; i += gridDim.x * blockDim.x) accumulate(acc, i);
-    }
-    if (*tp.n_tasks == 0) return;
-    Chunk<P, true> ck(smem + wid * Chunk<P, true>::kBytes, lane);
-    const int parts = item_parts(tp);
-
-    Item it;
-    while (next_item(tp, parts, lane, it)) {
-        bool again = it.n > 0;
-        for (int pass = 0; again; ++pass) {      // (the units of a pass as in k_grid)
-            again = false;
-            const bool report = it.blk == 0 && pass == 0;
-            ck.begin(tp, it.e0, it.n);
-            for (int j = 0; j >= 0;) {
-                if (j == ck.cnt) {
-                    if (!ck.next(tp, report)) break;
-                    j = 0;
-                }
-                const int key = ck.e[j].w, S = key_support(key), ch = key_chan(key);
-                const int nb = key < 0 ? 0 : (S * S + tp.slots - 1) / tp.slots;
-                int2 un = make_int2(0, 0);
-                if (it.blk < nb) {
-                    un = block_units(S, it.blk, nb);
-                    if (un.y - un.x > (pass + 1) * kUnitsMax) again = true;
-                    un = make_int2(un.x + pass * kUnitsMax, min(un.y, un.x + (pass + 1) * kUnitsMax));
-                }
-                if (un.x >= un.y) {
-                    ++j;
-                } else if ((ck.slow >> j) & 1) {
-                    const Staged e = ck.e[j];
-                    slow_entry<P, TS, COMP>(ck.g + j * P, S, un.x, un.y, e.x, table + (size_t)(unsigned)e.z * kPairBytes<TS>,
-                                            tp.N, lane, grid + (size_t)ch * tp.N * tp.N * P,
-                                            COMP ? errgrid + (size_t)ch * tp.N * tp.N * P : nullptr);
-                    ++j;
-                } else {
-                    j = jump_entries<P, TS, COMP>(ck, j, un.x, un.y, tp, report, table, grid, errgrid);
-                }
             }
         }
     }
@@ -452,21 +318,14 @@ template <int P, typename TS, bool COMP, bool SMALL>
 static int grid_launch(Grid& g, const Table& t, const WorkList& wl, const void* table, const AccumulateParams& acc,
                        cudaStream_t s)
 {
-    static int blocks_per_sm = 0, jump_blocks = 0;
+    static int blocks_per_sm = 0;
     if (blocks_per_sm == 0 &&
         (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks_per_sm, k_grid<P, TS, COMP, SMALL>, kWarps * 32, 0) != cudaSuccess ||
          blocks_per_sm < 1))
         blocks_per_sm = 1;
-    if (jump_blocks == 0 &&
-        (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&jump_blocks, k_grid_jumps<P, TS, COMP>, kWarps * 32, 0) != cudaSuccess ||
-         jump_blocks < 1))
-        jump_blocks = 1;
     k_grid<P, TS, COMP, SMALL><<<num_sms() * blocks_per_sm, kWarps * 32, 0, s>>>(
-        task_params(g, t, wl, wl.task_counter + 2, false), static_cast<const char*>(table), g.data, g.err);
+        task_params(g, t, wl, wl.task_counter + 2), static_cast<const char*>(table), g.data, g.err, acc);
     WG_LAUNCHED("k_grid");
-    k_grid_jumps<P, TS, COMP><<<num_sms() * jump_blocks, kWarps * 32, 0, s>>>(
-        task_params(g, t, wl, wl.task_counter + 3, true), static_cast<const char*>(table), g.data, g.err, acc);
-    WG_LAUNCHED("k_grid_jumps");
     return WG_OK;
 }
 
@@ -491,7 +350,7 @@ static int grid_dispatch(Grid& g, const Table& t, const WorkList& wl, const Accu
 template <int P>
 static int grid_impl(Grid& g, const Table& t, const WorkList& wl, cudaStream_t s)
 {
-    WG_CUDA(cudaMemsetAsync(wl.task_counter + 2, 0, 2 * sizeof(unsigned int), s));
+    WG_CUDA(cudaMemsetAsync(wl.task_counter + 2, 0, sizeof(unsigned int), s));
     // appended batches added their N_p terms at vis_compress
     AccumulateParams acc = {};
     if (!wl.append)

@@ -37,8 +37,6 @@ int num_sms();
 // ---- compile-time limits --------------------------------------------------------------
 constexpr int kMaxSupport = 1023;     // largest odd support
 constexpr int kMaxBeta = 64;
-// bit of a segment's seg_nblk: its footprints jump about, the gridder takes it in k_grid_jumps
-constexpr int kSegJumps = 1 << 30;
 constexpr int kTileRecords = 2048;    // records per preparation tile (rows x channels)
 constexpr int kSegLenMin = 32;        // gridded entries per gridder segment: range and default
 constexpr int kSegLenMax = 256;
@@ -125,11 +123,10 @@ struct WorkList {
     int2* runs = nullptr;
     float2* dacc = nullptr;               // [cap][P] degridding sums per entry (not in no-alloc views)
     // segments
-    int* seg_nblk = nullptr;              // task blocks | kSegJumps
+    int* seg_nblk = nullptr;              // task blocks
     int* seg_off = nullptr;               // [seg_cap + 1]
-    int* seg_offj = nullptr;              // [seg_cap + 1] the same of the tasks of kSegJumps segments alone
     // scalars and small arrays (device)
-    long long* scal = nullptr;            // [0] n_entries [1] n_tasks [2] n_seg [3] overflow [4] n_tasks of kSegJumps segments
+    long long* scal = nullptr;            // [0] n_entries [1] n_tasks [2] n_seg [3] overflow
     int* chan_base = nullptr;             // [C + 1]
     double* norm_priv = nullptr;          // [kNormSlots][C][P]
     double* norm_batch = nullptr;         // [C][P]

@@ -128,7 +128,6 @@ extern "C" int grid_vis_noalloc(const wg_grid_view* view, const wg_table* th, co
     w.runs = cv.take<int2>(cap);
     w.seg_nblk = cv.take<int>(w.seg_cap);
     w.seg_off = cv.take<int>(w.seg_cap + 1);
-    w.seg_offj = cv.take<int>(w.seg_cap + 1);
     w.scal = cv.take<long long>(8);
     w.chan_base = cv.take<int>(C + 1);
     w.norm_priv = cv.take<double>((int64_t)kNormSlots * C * P);

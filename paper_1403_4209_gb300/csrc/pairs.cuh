@@ -104,7 +104,6 @@ struct TaskParams {
     const int4* entries;
     const float2* gamma;
     const int* seg_off;
-    const int* seg_nblk;
     const long long* scal;
     const long long* n_tasks;
     const int* supports;
@@ -123,11 +122,6 @@ struct TaskParams {
 //   z: the first pair of its sub-kernel in the paired table
 //   w: key, support << 16 | grid channel; -1: rejected by the bounds checks
 typedef int4 Staged;
-// A move of the footprint by one column or row: every pair's sample offset (in pairs) shifts by x; the
-// one class column (or row) that left the footprint wraps to the other side, its offset shifts by y;
-// z: what is added to a wrapped pair's first pixel (column | row << 16);
-// w: the class | the byte selector of its axis in a packed class << 16.
-typedef int4 Move;
 __device__ __forceinline__ int key_support(int key) { return key >> 16; }
 __device__ __forceinline__ int key_chan(int key) { return key & 0xFFFF; }
 
@@ -179,21 +173,6 @@ __device__ __forceinline__ void place_classes(unsigned (&toff)[NU], int (*cls)[3
     }
 }
 
-// Takes a lane's pairs through one move; bit u of the result: unit u's pair wraps.
-template <int NU, int PB>
-__device__ __forceinline__ unsigned move_classes(unsigned (&toff)[NU], const int (*cls)[32], const Move& m, int lane)
-{
-    unsigned wraps = 0;
-    const int shift = m.x * PB, wrap = m.y * PB, c = m.w & 0xFFFF, sel = m.w >> 16;
-#pragma unroll
-    for (int u = 0; u < NU; ++u) {
-        const bool w = (int)__byte_perm(cls[u][lane], 0, sel) == c;
-        toff[u] += w ? wrap : shift;
-        wraps |= w ? 1u << u : 0u;
-    }
-    return wraps;
-}
-
 // Places a pair of class cl (column | row << 16) in the footprint of entry E: its column | row << 16 there.  Each
 // half of cl + E.y is less than twice its modulus, so that the smaller of it and it less the modulus (as an unsigned
 // 16-bit number) is the remainder; minus_sh = minus_moduli(S, H).
@@ -223,34 +202,31 @@ __device__ __forceinline__ int2 block_units(int S, int blk, int nb)
 }
 
 // A warp's walk over the entries of its work item, 32 at a time.  Each lane stages one entry: its
-// checks, residues, sub-kernel and the move from its predecessor are worked out once, in parallel, and
-// the warp keeps bit masks of the entries at which something changes, so that the record loops run
+// checks, residues and sub-kernel are worked out once, in parallel, and the warp keeps bit masks of the entries at which something changes, so that the record loops run
 // over stretches without a test.  The next 32 entries are on their way (cp.async) meanwhile.
 // With GAMMA the weighted visibilities are staged too.
 template <int P, bool GAMMA>
 struct Chunk {
     static constexpr int kG = GAMMA ? 32 * P * (int)sizeof(float2) : 0;
-    static constexpr int kM = GAMMA ? 32 : 0;
-    static constexpr int kBytes = (64 + kM) * (int)sizeof(int4) + 2 * kG + (2 * kUnitsMax + 1) * 32 * (int)sizeof(int);
+    static constexpr int kBytes = 64 * (int)sizeof(int4) + 2 * kG + (3 * kUnitsMax + 1) * 32 * (int)sizeof(int);
     int4* raw_e;             // [32] as copied
     Staged* e;               // [32]
-    Move* m;                 // [32] from the entry's predecessor (entries of mv that are not of kc; the gridder's)
     float2* raw_g;           // [32][P]
     float2* g;               // [32][P] weighted visibilities
     unsigned* z;             // [32] the entries' z again
     int (*cls)[32];          // [kUnitsMax][32] the lanes' classes
     int (*cur)[32];          // [kUnitsMax][32] the first pixels of the pairs they hold
+    int (*nxt)[32];          // [kUnitsMax][32] the first pixels after a move (the gridder's)
     int lane;
     int e0, left, cnt;       // the chunk's first entry in the lists, entries from there to the item's end, its entries
-    unsigned kc;             // entries that start a run: another support or channel, a jump (of the gridder's), or around
-                             // a slow one
+    unsigned kc;             // entries that start a run: another support or channel, or around a slow one
     unsigned mv;             // entries whose footprint differs from their predecessor's (and kc)
     unsigned slow;           // entries with an infinite or NaN visibility
 
     __device__ __forceinline__ Chunk(unsigned char* base, int lane_)
-        : raw_e(reinterpret_cast<int4*>(base)), e(raw_e + 32), m(e + 32), raw_g(reinterpret_cast<float2*>(m + kM)),
+        : raw_e(reinterpret_cast<int4*>(base)), e(raw_e + 32), raw_g(reinterpret_cast<float2*>(e + 32)),
           g(raw_g + kG / sizeof(float2)), z(reinterpret_cast<unsigned*>(g + kG / sizeof(float2))),
-          cls(reinterpret_cast<int (*)[32]>(z + 32)), cur(cls + kUnitsMax), lane(lane_)
+          cls(reinterpret_cast<int (*)[32]>(z + 32)), cur(cls + kUnitsMax), nxt(cls + 2 * kUnitsMax), lane(lane_)
     {
     }
 
@@ -320,20 +296,7 @@ struct Chunk {
             qk = pkey;
             qf = last.x;
         }
-        bool k = s.w != qk || sl || qs;
-        if constexpr (GAMMA) {
-            // the move from the predecessor
-            const int S = key_support(s.w), H = (S + 1) >> 1;
-            const int dx = (s.x & 0xFFFF) - (qf & 0xFFFF), dy = (s.x >> 16) - (qf >> 16);
-            const bool along_x = dy == 0;
-            const int d = dx + dy, md = along_x ? S : H, step = along_x ? 1 : S;
-            const int cn = along_x ? s.y & 0xFFFF : s.y >> 16;             // (-origin) mod md
-            const int o = cn ? md - cn : 0;                                // origin mod md
-            const int c = d > 0 ? (o ? o - 1 : md - 1) : o;                // the class that wraps
-            k = k || abs(dx) + abs(dy) > 1;
-            m[lane] = make_int4(-d * step, d * (md - 1) * step, along_x ? d * S : d * H * 65536,
-                                c | ((along_x ? 0x4410 : 0x4432) << 16));
-        }
+        const bool k = s.w != qk || sl || qs;
         kc = __ballot_sync(0xffffffffu, in && k);
         mv = __ballot_sync(0xffffffffu, in && (k || s.x != qf));
         e[lane] = s;
@@ -359,7 +322,6 @@ struct Chunk {
 // segment is cut into parts, so that every warp has something to do (17 tasks on 2432 warps: 204 -> 25 us).
 struct Item {
     int blk, e0, n;          // block of the footprint, first entry, entries
-    int seg;                 // its segment
 };
 
 __device__ __forceinline__ int item_parts(const TaskParams& tp)
@@ -386,7 +348,6 @@ __device__ __forceinline__ bool next_item(const TaskParams& tp, int parts, int l
         hi = min(hi, lo + step);
     }
     it.blk = (int)t - __ldg(&tp.seg_off[lo]);
-    it.seg = lo;
     it.e0 = lo * tp.seg_len;
     it.n = (int)min((long long)tp.seg_len, tp.scal[0] - it.e0);
     if (parts > 1) {
@@ -398,11 +359,10 @@ __device__ __forceinline__ bool next_item(const TaskParams& tp, int parts, int l
     return true;
 }
 
-// jumps: the tasks of the segments whose footprints jump about, not all
-inline TaskParams task_params(const Grid& g, const Table& t, const WorkList& wl, unsigned* counter, bool jumps)
+inline TaskParams task_params(const Grid& g, const Table& t, const WorkList& wl, unsigned* counter)
 {
-    return {wl.entries, wl.gamma, jumps ? wl.seg_offj : wl.seg_off, wl.seg_nblk, wl.scal, wl.scal + (jumps ? 4 : 1), t.supports_d, t.offsets_d, t.poffsets_d, g.n,     t.K,
-            g.n_chan,    t.beta * t.beta, t.n_samples, wl.seg_len,   wl.slots,    counter,      wl.scal + 3};
+    return {wl.entries, wl.gamma, wl.seg_off,         wl.scal,     wl.scal + 1, t.supports_d, t.offsets_d, t.poffsets_d, g.n, t.K,
+            g.n_chan,   t.beta * t.beta, t.n_samples, wl.seg_len,  wl.slots,    counter,      wl.scal + 3};
 }
 
 }  // namespace

@@ -1160,10 +1160,9 @@ __global__ void k_carry(const float2* __restrict__ carry_q, const int* __restric
     atomicMax(reinterpret_cast<int*>(&runs[dst]) + 1, last);
 }
 
-// per segment, the number of task blocks of its largest support (one warp a segment), and whether its footprints jump
-// about: one entry in `few` at least does not lie within one column or row of its predecessor; sets the segment count
+// per segment, the number of task blocks of its largest support (one warp a segment); sets the segment count
 __global__ void k_segments(const int4* __restrict__ entries, long long* __restrict__ scal,
-                           const int* __restrict__ supports, int K, int seg_len, int slots, int few,
+                           const int* __restrict__ supports, int K, int seg_len, int slots,
                            int* __restrict__ seg_nblk)
 {
     const long long n = scal[0], n_seg = (n + seg_len - 1) / seg_len;
@@ -1173,58 +1172,41 @@ __global__ void k_segments(const int4* __restrict__ entries, long long* __restri
     for (long long g = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; g < n_seg; g += n_warps) {
         const int len = (int)min((long long)seg_len, n - g * seg_len);
         const int4* e = entries + g * seg_len;
-        int nb = 0, jumps = 0;
+        int nb = 0;
         for (int i = lane; i < len; i += 32) {
-            const int4 E = e[i], Q = e[max(i - 1, 0)];
-            const int k = E.w & 0xFFF;
+            const int k = e[i].w & 0xFFF;
             nb = max(nb, (k < K) ? nblk_of(__ldg(&supports[k]), slots) : 1);
-            jumps += E.w != Q.w || abs((E.x & 0xFFFF) - (Q.x & 0xFFFF)) + abs((E.x >> 16) - (Q.x >> 16)) > 1;
         }
         nb = __reduce_max_sync(0xffffffffu, nb);
-        jumps = __reduce_add_sync(0xffffffffu, jumps);
-        if (lane == 0) seg_nblk[g] = nb | (few * jumps >= len ? kSegJumps : 0);
+        if (lane == 0) seg_nblk[g] = nb;
     }
 }
 
 // exclusive scan of the segments' task counts (one block; kScan segments a thread and step, as above)
 __global__ void __launch_bounds__(1024) k_seg_scan(const int* __restrict__ seg_nblk, int* __restrict__ seg_off,
-                                                   int* __restrict__ seg_offj, long long* __restrict__ scal, unsigned long long* __restrict__ stats)
+                                                   long long* __restrict__ scal, unsigned long long* __restrict__ stats)
 {
     __shared__ int warp_tot[32];
     const long long n_seg = scal[2];
-    int carry = 0, carry_j = 0;
+    int carry = 0;
     for (long long base = 0; base < n_seg; base += (long long)blockDim.x * kScan) {
         const long long t0 = base + (long long)threadIdx.x * kScan;
-        int v[kScan], sum = 0, sum_j = 0, total;
+        int v[kScan], sum = 0, total;
 #pragma unroll
         for (int i = 0; i < kScan; ++i) v[i] = (t0 + i < n_seg) ? seg_nblk[t0 + i] : 0;
 #pragma unroll
-        for (int i = 0; i < kScan; ++i) {
-            sum_j += v[i] & kSegJumps ? v[i] & ~kSegJumps : 0;
-            sum += v[i] & ~kSegJumps;
-        }
-        int at_j = carry_j;
-        if (__syncthreads_or(sum_j)) {
-            at_j += block_inclusive(sum_j, warp_tot, total) - sum_j;
-            carry_j += total;
-        }
+        for (int i = 0; i < kScan; ++i) sum += v[i];
         int at = carry + block_inclusive(sum, warp_tot, total) - sum;
 #pragma unroll
         for (int i = 0; i < kScan; ++i) {
-            if (t0 + i < n_seg) {
-                seg_off[t0 + i] = at;
-                seg_offj[t0 + i] = at_j;
-            }
-            at += v[i] & ~kSegJumps;
-            at_j += v[i] & kSegJumps ? v[i] & ~kSegJumps : 0;
+            if (t0 + i < n_seg) seg_off[t0 + i] = at;
+            at += v[i];
         }
         carry += total;
     }
     if (threadIdx.x == 0) {
         seg_off[n_seg] = carry;
-        seg_offj[n_seg] = carry_j;
         scal[1] = carry;
-        scal[4] = carry_j;
         stats[ST_TASKS] = (unsigned long long)carry;
     }
 }
@@ -1382,9 +1364,9 @@ static int prep_impl(const Table& t, const Grid& g, const wg_vis_in& in, int fla
 int launch_plan(const Table& t, WorkList& wl, cudaStream_t s)
 {
     k_segments<<<num_sms() * 8, 256, 0, s>>>(wl.entries, wl.scal, t.supports_d, t.K, wl.seg_len, wl.slots,
-                                             wl.P == 4 ? 6 : 2, wl.seg_nblk);
+                                             wl.seg_nblk);
     WG_LAUNCHED("k_segments");
-    k_seg_scan<<<1, 1024, 0, s>>>(wl.seg_nblk, wl.seg_off, wl.seg_offj, wl.scal, wl.stats);
+    k_seg_scan<<<1, 1024, 0, s>>>(wl.seg_nblk, wl.seg_off, wl.scal, wl.stats);
     WG_LAUNCHED("k_seg_scan");
     return WG_OK;
 }
