@@ -292,10 +292,10 @@ __global__ void __launch_bounds__(kWarps * 32, P == 4 ? (SMALL ? 5 : 4) : P == 2
                     ++j;
                     continue;
                 }
-                // the variant for small supports saves idle units at one and two polarisations (28 against 33 us on
-                // 127 k entries of support 7); at four, and with compensation, its code costs more in the
-                // instruction cache (21.1 against 20.5 ms on 21 M entries of supports 9..65)
-                if (!SMALL && (P == 4 || COMP || un.y - un.x > 2))
+                // the variant for one or two units (supports up to 9, and the last block of some others) saves idle ones:
+                // support 7 beside 31 in the table, P = 4, 2.31 -> 1.30 ms on 3.4 M entries (single points 1.78); 116 M
+                // records of supports 9..65, P = 4, 20.5 -> 20.2 ms; support 7 at P = 1, 33 -> 28 us on 127 k entries
+                if (!SMALL && un.y - un.x > 2)
                     j = run_entries<P, TS, COMP, kUnitsMax>(ck, j, S, ch, un, tp, report, table, grid, errgrid);
                 else
                     j = run_entries<P, TS, COMP, 2>(ck, j, S, ch, un, tp, report, table, grid, errgrid);
