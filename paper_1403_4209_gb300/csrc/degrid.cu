@@ -290,7 +290,7 @@ __global__ void __launch_bounds__(kWarps * 32, P == 4 ? 4 : 5) k_degrid_sum(Task
                     j = ck.run_end(j);
                     continue;
                 }
-                // (at P = 4: support 7, 4288 -> 2950 us on 6.9 M entries, where all four units took as long as single points)
+                // (at P = 4: support 7, 4288 -> 2950 us on 13.8 M entries, where all four units took as long as single points)
                 if (un.y - un.x > 2)
                     j = degrid_entries<P, kUnitsMax>(ck, j, S, ch, un, tp, report, red, table, grid, acc);
                 else

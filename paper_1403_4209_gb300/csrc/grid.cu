@@ -293,7 +293,7 @@ __global__ void __launch_bounds__(kWarps * 32, P == 4 ? (SMALL ? 5 : 4) : P == 2
                     continue;
                 }
                 // the variant for one or two units (supports up to 9, and the last block of some others) saves idle ones:
-                // support 7 beside 31 in the table, P = 4, 2.31 -> 1.30 ms on 3.4 M entries (single points 1.78); 116 M
+                // support 7 beside 31 in the table, P = 4, 2.31 -> 1.30 ms on 13.8 M entries (single points 1.78); 116 M
                 // records of supports 9..65, P = 4, 20.5 -> 20.2 ms; support 7 at P = 1, 33 -> 28 us on 127 k entries
                 if (!SMALL && un.y - un.x > 2)
                     j = run_entries<P, TS, COMP, kUnitsMax>(ck, j, S, ch, un, tp, report, table, grid, errgrid);
