@@ -387,8 +387,8 @@ int grid_autotune(wg_grid* grid, const wg_table* table, wg_worklist* wl, const w
  * eps'_p = eps_p / W_p (0 where W_p = 0); robust: eps'_p = eps_p / (1 + W_p f_p^2) with
  * f_p^2 = (5 10^-robust)^2 sum eps_p (1 - f_p) / sum_cells W_p^2.  Records that are not
  * griddable keep eps.  weight_out: device float [n_rows][n_chan][n_pol], may alias in->weight.
- * Allocates and frees a float density grid of (grid channels) x N^2 x n_pol and 4 bytes per
- * record on `stream` (stream-ordered).  Errors: INVALID_ARG, SHAPE, OOM, CUDA. */
+ * Allocates and frees a float density grid of (grid channels) x N^2 x n_pol on `stream`
+ * (stream-ordered), and 4 bytes per record where there is memory for them (without, every record is placed twice).  Errors: INVALID_ARG, SHAPE, OOM, CUDA. */
 int vis_weight(const wg_grid* grid, const wg_table* table, const wg_vis_in* in, int32_t scheme,
                double robust, int32_t flags, float* weight_out, void* stream);
 

@@ -1426,7 +1426,7 @@ __device__ __forceinline__ void add_exact(float& s, float& e, float x)
     s = t;
 }
 
-// The densities, each record's cell (for k_reweight, which then need not place it again), and sum eps (1 - f).
+// The densities, each record's cell (cells not null: for k_reweight, which then need not place it again), and sum eps (1 - f).
 template <int P, typename IDX>
 __global__ void __launch_bounds__(256) k_density(const double* __restrict__ uvw, const double* __restrict__ lam_inv,
                                                  const double* __restrict__ sc, const float* __restrict__ lam_f,
@@ -1446,11 +1446,11 @@ __global__ void __launch_bounds__(256) k_density(const double* __restrict__ uvw,
         const int4 info = place(uvw, (int64_t)row, row_f(uvw, (int64_t)row), lam_inv, sc, ch, lam_f[ch], sc_f[ch], flag,
                                 (int64_t)rec, P, pp).info;
         if (!((info.w >> kBitGd) & 1)) {
-            cells[rec] = kNoCell;
+            if (cells) cells[rec] = kNoCell;
             continue;
         }
         const unsigned cell = cell_of(info, pp.supports);
-        cells[rec] = cell;
+        if (cells) cells[rec] = cell;
         float w[P], wf[P];
         load_weights<P>(weight, flag, rec, vec, w, wf);
         float* d = dens + (((size_t)(pp.interleave ? 0 : ch) * pp.N + (cell >> 16)) * pp.N + (cell & 0xFFFF)) * P;
@@ -1539,8 +1539,12 @@ __device__ __forceinline__ float robust_weight(float w, float W, double f2, floa
     return (float)((double)w / (1.0 + (double)W * f2));
 }
 
-template <int P, typename IDX>
-__global__ void __launch_bounds__(256) k_reweight(const unsigned* __restrict__ cells, const float* __restrict__ weight,
+// KEPT: k_density kept the records' cells; if there was no memory for them, they are placed again
+template <int P, typename IDX, bool KEPT>
+__global__ void __launch_bounds__(256) k_reweight(const unsigned* __restrict__ cells, const double* __restrict__ uvw,
+                                                  const double* __restrict__ lam_inv, const double* __restrict__ sc,
+                                                  const float* __restrict__ lam_f, const float* __restrict__ sc_f,
+                                                  const uint8_t* __restrict__ flag, const float* __restrict__ weight,
                                                   int64_t rows, PlaceParams pp, const float* __restrict__ dens,
                                                   const double* __restrict__ sums, int scheme, double robust_f0,
                                                   float* __restrict__ out)
@@ -1556,7 +1560,16 @@ __global__ void __launch_bounds__(256) k_reweight(const unsigned* __restrict__ c
         f2l[p] = (float)(f2[p] - (double)f2h[p]);
     }
     for (IDX rec = (IDX)blockIdx.x * blockDim.x + threadIdx.x; rec < n; rec += step) {
-        const unsigned cell = cells[rec];
+        unsigned cell;
+        if constexpr (KEPT) {
+            cell = cells[rec];
+        } else {
+            const IDX row = rec / C;
+            const int ch = (int)(rec - row * C);
+            const int4 info = place(uvw, (int64_t)row, row_f(uvw, (int64_t)row), lam_inv, sc, ch, lam_f[ch], sc_f[ch], flag,
+                                    (int64_t)rec, P, pp).info;
+            cell = (info.w >> kBitGd) & 1 ? cell_of(info, pp.supports) : kNoCell;
+        }
         float w[P];
         if (vec && P == 4) {
             const float4 a = *(reinterpret_cast<const float4*>(weight) + rec);
@@ -1597,9 +1610,8 @@ static int weight_impl(const Table& t, const Grid& g, const wg_vis_in& in, int s
     pp.flag_vec = (reinterpret_cast<uintptr_t>(in.flag) % P) == 0;
     const int gc = pp.interleave ? 1 : C;
     const int64_t n_cells = (int64_t)gc * g.n * g.n;
-    // the densities, the channel scales, the sums, and each record's cell
-    const size_t bytes = sizeof(float) * (size_t)n_cells * P + sizeof(double) * (4 * C + 2 * P) +
-                         sizeof(unsigned) * (size_t)(rows * C);
+    // the densities, the channel scales and the sums
+    const size_t bytes = sizeof(float) * (size_t)n_cells * P + sizeof(double) * (4 * C + 2 * P);
     void* scratch = nullptr;
     if (cudaMallocAsync(&scratch, bytes, s) != cudaSuccess) {
         cudaGetLastError();
@@ -1611,7 +1623,12 @@ static int weight_impl(const Table& t, const Grid& g, const wg_vis_in& in, int s
     float* lam_f = reinterpret_cast<float*>(sums + 2 * P);
     float* sc_f = lam_f + C;
     float* dens = reinterpret_cast<float*>(lam_inv + (4 * C + 2 * P));   // 4 C + 2 P is even: 16-byte aligned
-    unsigned* cells = reinterpret_cast<unsigned*>(dens + (size_t)n_cells * P);
+    // each record's cell, if there is memory for them
+    unsigned* cells = nullptr;
+    if (rows > 0 && cudaMallocAsync((void**)&cells, sizeof(unsigned) * (size_t)(rows * C), s) != cudaSuccess) {
+        cudaGetLastError();
+        cells = nullptr;
+    }
     const int vec = reinterpret_cast<uintptr_t>(in.weight) % (4 * P) == 0 && pp.flag_vec;
     int rc = WG_OK;
     if (cudaMemsetAsync(dens, 0, sizeof(float) * (size_t)n_cells * P, s) != cudaSuccess ||
@@ -1632,7 +1649,12 @@ static int weight_impl(const Table& t, const Grid& g, const wg_vis_in& in, int s
                     k_density_sq<P><<<blocks, 256, 0, s>>>(dens, n_cells, sums);
                     WG_LAUNCHED("k_density_sq");
                 }
-                k_reweight<P, IDX><<<blocks, 256, 0, s>>>(cells, in.weight, rows, pp, dens, sums, scheme, f0, out);
+                if (cells)
+                    k_reweight<P, IDX, true><<<blocks, 256, 0, s>>>(cells, in.uvw, lam_inv, sc, lam_f, sc_f, in.flag, in.weight, rows,
+                                                                    pp, dens, sums, scheme, f0, out);
+                else
+                    k_reweight<P, IDX, false><<<blocks, 256, 0, s>>>(cells, in.uvw, lam_inv, sc, lam_f, sc_f, in.flag, in.weight, rows,
+                                                                     pp, dens, sums, scheme, f0, out);
                 WG_LAUNCHED("k_reweight");
                 return WG_OK;
             };
@@ -1640,6 +1662,7 @@ static int weight_impl(const Table& t, const Grid& g, const wg_vis_in& in, int s
         }
         if (rc == WG_OK && cudaGetLastError() != cudaSuccess) rc = fail(WG_E_CUDA, "weighting kernels failed to launch");
     }
+    if (cells) cudaFreeAsync(cells, s);
     cudaFreeAsync(scratch, s);
     return rc;
 }
