@@ -219,9 +219,14 @@ typedef struct wg_table_info {
     int32_t reserved;
     const void* data_lp;      /* device complex bf16/f16 [n_samples], or NULL for WG_F32 */
 } wg_table_info;
-/* Sizes and device pointers (owned by the table) of C-1 .. C-3 (Sec. 4.2.2).
- * Errors: INVALID_ARG. */
+/* Sizes and device pointers (owned by the table) of C-1 .. C-3 (Sec. 4.2.2).  The table keeps C-1 as the
+ * gridder reads it, 8 (1 + 1/S) bytes a sample of a plane of support S (and 4 (1 + 1/S) more in a reduced
+ * store); the first call makes the copies in the order given here, 8 bytes a sample and 4, and synchronises the
+ * device.  Errors: INVALID_ARG, OOM, CUDA. */
 int table_info(const wg_table* table, wg_table_info* info);
+/* The same (C-2 and C-3 of Sec. 4.2.2) without C-1: data and data_lp are NULL and nothing is made.
+ * Errors: INVALID_ARG. */
+int table_params(const wg_table* table, wg_table_info* info);
 /* Copies C-1 (complex float32, interleaved), C-3 and C-2 (Sec. 4.2.2) to caller-owned host
  * buffers sized from table_info; any pointer may be NULL.  Synchronises the device.
  * Errors: INVALID_ARG, CUDA. */

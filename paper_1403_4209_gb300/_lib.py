@@ -86,6 +86,7 @@ def _load():
         "table_destroy": (c_i32, [c_vp]),
         "table_set_store": (c_i32, [c_vp, c_i32]),
         "table_info": (c_i32, [c_vp, P(TableInfo)]),
+        "table_params": (c_i32, [c_vp, P(TableInfo)]),
         "table_copy_to_host": (c_i32, [c_vp, c_vp, c_vp, c_vp, c_vp]),
         "worklist_create": (c_i32, [c_i64, c_i32, c_i32, P(c_vp)]),
         "worklist_create2": (c_i32, [c_i64, c_i64, c_i32, c_i32, P(c_vp)]),

@@ -118,7 +118,7 @@ class ConvTable:
     def __init__(self, handle):
         self._h = handle
         info = TableInfo()
-        check(lib.table_info(self._h, ctypes.byref(info)), "table_info")
+        check(lib.table_params(self._h, ctypes.byref(info)), "table_params")
         self.n_wplanes = info.n_wplanes
         self.oversample = info.oversample
         self.taper_support = info.taper_support

@@ -233,9 +233,9 @@ int table_destroy(wg_table* h)
     return WG_OK;
 }
 
-int table_info(const wg_table* h, wg_table_info* info)
+int table_params(const wg_table* h, wg_table_info* info)
 {
-    if (!h || !info) return fail(WG_E_INVALID_ARG, "table_info: null argument");
+    if (!h || !info) return fail(WG_E_INVALID_ARG, "table_params: null argument");
     const Table& t = h->t;
     info->n_wplanes = t.K;
     info->oversample = t.beta;
@@ -244,12 +244,23 @@ int table_info(const wg_table* h, wg_table_info* info)
     info->n_samples = t.n_samples;
     info->w_max = t.w_max;
     info->du = t.du;
-    info->data = t.data;
+    info->data = nullptr;
     info->zeta = t.zeta;
     info->supports = t.supports_d;
     info->offsets = t.offsets_d;
     info->store_dtype = t.store;
     info->reserved = 0;
+    info->data_lp = nullptr;
+    return WG_OK;
+}
+
+int table_info(const wg_table* h, wg_table_info* info)
+{
+    if (!h || !info) return fail(WG_E_INVALID_ARG, "table_info: null argument");
+    Table& t = const_cast<Table&>(h->t);             // the samples in their order are made when first asked for
+    if (int rc = table_samples(t)) return rc;
+    table_params(h, info);
+    info->data = t.data;
     info->data_lp = t.data_lp;
     return WG_OK;
 }
@@ -258,7 +269,8 @@ int table_copy_to_host(const wg_table* h, float* data, double* zeta, int32_t* su
 {
     if (!h) return fail(WG_E_INVALID_ARG, "table_copy_to_host: null table");
     const Table& t = h->t;
-    if (data) WG_CUDA(cudaMemcpy(data, t.data, sizeof(float2) * t.n_samples, cudaMemcpyDeviceToHost));
+    if (data)
+        if (int rc = table_to_host(t, data)) return rc;
     if (zeta) WG_CUDA(cudaMemcpy(zeta, t.zeta, sizeof(double) * t.K * t.beta * t.beta, cudaMemcpyDeviceToHost));
     if (supports) std::memcpy(supports, t.supports.data(), sizeof(int) * t.K);
     if (offsets) std::memcpy(offsets, t.offsets.data(), sizeof(int) * t.K);

@@ -74,12 +74,13 @@ struct Table {
     int K = 0, beta = 0, s0 = 0, max_support = 0;
     double w_max = 0, du = 0;
     int64_t n_samples = 0;
-    float2* data = nullptr;               // C-1, complex float32
-    int store = WG_F32;                   // samples the gridder reads
-    void* data_lp = nullptr;              // C-1 as complex bf16 / f16 (store != WG_F32)
-    // C-1 as the gridder and the degridder read it: sample pairs {re, re', im, im'} (pairs.cuh)
+    // C-1 as the gridder and the degridder read it: sample pairs {re, re', im, im'} (pairs.cuh), complex float32
     float4* pairs = nullptr;
+    int store = WG_F32;                   // samples the gridder reads
     void* pairs_lp = nullptr;             // the same as bf16 / f16 (store != WG_F32)
+    // C-1 in the order of its definition, once a caller has asked for it (table_samples)
+    float2* data = nullptr;
+    void* data_lp = nullptr;              // (store != WG_F32)
     unsigned* poffsets_d = nullptr;       // [K] first pair of each plane
     int64_t n_pairs = 0;
     double* zeta = nullptr;               // C-3 [K beta^2]
@@ -179,6 +180,10 @@ int import_table(int K, int beta, double w_max, double du, int s0, const int* su
                  const double* data, const double* zeta, Table& t);
 int free_table(Table& t);
 int set_table_store(Table& t, int store);
+// fills data and data_lp; synchronises the device the first time
+int table_samples(Table& t);
+// copies C-1 in the order of its definition to `data` (n_samples complex floats)
+int table_to_host(const Table& t, float* data);
 
 // psi_0(c, x) from its even Legendre coefficients a[0..n): sum_m a_m P_2m(x), by the
 // three-term Legendre recurrence.

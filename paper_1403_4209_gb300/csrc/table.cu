@@ -16,6 +16,7 @@
 //   6. zeta = sum of real parts of each sub-kernel (eq. "sum"), in FP64 before rounding to FP32.
 #include <cmath>
 #include <cstdio>
+#include <mutex>
 #include <vector>
 
 #include <cuda_bf16.h>
@@ -103,18 +104,19 @@ __global__ void k_support_radius(const double2* C, int M, double thr2, int* radi
     if ((threadIdx.x & 31) == 0 && r >= 0) atomicMax(radius, r);
 }
 
-// one block per sub-kernel: trim, normalise, round to float, and zeta
-__global__ void k_trim(const double2* C, int M, int beta, int S, const double* normp, float2* out,
+// one block per sub-kernel: trim, normalise, round to float, and zeta.  The samples go where the gridder and the degridder
+// read them: H = (S + 1) / 2 rows of S pairs {re, re', im, im'} (pairs.cuh), the second row past the last one zero.
+__global__ void k_trim(const double2* C, int M, int beta, int S, const double* normp, float4* out,
                        double* zeta)
 {
     __shared__ double red[256];
     const int sub = blockIdx.x;                      // (fv - lo) * beta + (fu - lo)
     const int lo = -((beta - 1) / 2);
     const int fv = sub / beta + lo, fu = sub % beta + lo;
-    const int h = (S - 1) / 2;
+    const int h = (S - 1) / 2, H = (S + 1) / 2;
     const double inv = 1.0 / *normp;
     double acc = 0.0;
-    float2* dst = out + (int64_t)sub * S * S;
+    float* dst = reinterpret_cast<float*>(out + (int64_t)sub * S * H);
     for (int s = threadIdx.x; s < S * S; s += blockDim.x) {
         int i = s / S, j = s - i * S;
         int ov = beta * (i - h) - fv, ou = beta * (j - h) - fu;
@@ -126,7 +128,11 @@ __global__ void k_trim(const double2* C, int M, int beta, int S, const double* n
             re = v.x * sg;
             im = v.y * sg;
         }
-        dst[s] = make_float2((float)re, (float)im);
+        const int second = i >= H ? 1 : 0;
+        float* d = dst + 4 * ((i - second * H) * S + j);
+        d[second] = (float)re;
+        d[2 + second] = (float)im;
+        if (i == H - 1) d[1] = d[3] = 0.f;               // row S
         acc += re;
     }
     red[threadIdx.x] = acc;
@@ -145,51 +151,88 @@ static int default_nk(int s_max)
     return n;
 }
 
-// C-1 as pairs (pairs.cuh): plane k (blockIdx.y), per sub-kernel H = (S + 1) / 2 rows of S pairs; pair
-// (i, c) holds the samples of rows i and i + H in column c (zero past the last row).
-__global__ void k_table_pairs(const float2* __restrict__ src, const int* __restrict__ supports,
-                              const int* __restrict__ offsets, const unsigned* __restrict__ poffsets, int beta2, int store,
-                              void* __restrict__ dst)
-{
-    const int k = blockIdx.y, S = supports[k], H = (S + 1) / 2;
-    const float2* s = src + offsets[k];
-    const int64_t total = (int64_t)beta2 * S * H;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t sub = i / (S * H);
-        const int r = (int)(i - sub * (S * H));
-        const float2* p = s + sub * S * S + r;
-        const float2 a = p[0];
-        const float2 b = r + H * S < S * S ? p[H * S] : make_float2(0.f, 0.f);
-        const int64_t o = (int64_t)poffsets[k] + i;
-        if (store == WG_F32) {
-            reinterpret_cast<float4*>(dst)[o] = make_float4(a.x, b.x, a.y, b.y);
-        } else if (store == WG_BF16) {
-            reinterpret_cast<__nv_bfloat162*>(dst)[2 * o] = __floats2bfloat162_rn(a.x, b.x);
-            reinterpret_cast<__nv_bfloat162*>(dst)[2 * o + 1] = __floats2bfloat162_rn(a.y, b.y);
-        } else {
-            reinterpret_cast<__half2*>(dst)[2 * o] = __floats2half2_rn(a.x, b.x);
-            reinterpret_cast<__half2*>(dst)[2 * o + 1] = __floats2half2_rn(a.y, b.y);
-        }
-    }
-}
-
-static int fill_pairs(const Table& t, int store, void* dst, cudaStream_t s)
-{
-    k_table_pairs<<<dim3(num_sms(), t.K), 256, 0, s>>>(t.data, t.supports_d, t.offsets_d, t.poffsets_d, t.beta * t.beta,
-                                                      store, dst);
-    WG_LAUNCHED("k_table_pairs");
-    return WG_OK;
-}
-
-__global__ void k_table_lp(const float2* __restrict__ src, int64_t n, int store, void* __restrict__ dst)
+// the pairs as bf16 or f16: the two real parts, the two imaginary parts
+__global__ void k_pairs_lp(const float4* __restrict__ src, int64_t n, int store, uint2* __restrict__ dst)
 {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    const float2 v = src[i];
-    if (store == WG_BF16)
-        reinterpret_cast<__nv_bfloat162*>(dst)[i] = __floats2bfloat162_rn(v.x, v.y);
-    else
-        reinterpret_cast<__half2*>(dst)[i] = __floats2half2_rn(v.x, v.y);
+    const float4 v = src[i];
+    if (store == WG_BF16) {
+        reinterpret_cast<__nv_bfloat162*>(dst)[2 * i] = __floats2bfloat162_rn(v.x, v.y);
+        reinterpret_cast<__nv_bfloat162*>(dst)[2 * i + 1] = __floats2bfloat162_rn(v.z, v.w);
+    } else {
+        reinterpret_cast<__half2*>(dst)[2 * i] = __floats2half2_rn(v.x, v.y);
+        reinterpret_cast<__half2*>(dst)[2 * i + 1] = __floats2half2_rn(v.z, v.w);
+    }
+}
+
+// C-1 in the order of its definition from the pairs: plane k (blockIdx.y), sample i of its beta^2 S^2.  Bits are
+// copied: T is a component as stored (float: 32 bits, unsigned short: bf16 or f16).
+template <typename T>
+__global__ void k_samples(const T* __restrict__ pairs, const int* __restrict__ supports, const int* __restrict__ offsets,
+                          const unsigned* __restrict__ poffsets, int beta2, T* __restrict__ dst)
+{
+    const int k = blockIdx.y, S = supports[k], H = (S + 1) / 2;
+    const int64_t total = (int64_t)beta2 * S * S;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t sub = i / (S * S);
+        const int s = (int)(i - sub * (S * S)), second = s >= H * S ? 1 : 0;
+        const T* p = pairs + 4 * ((int64_t)poffsets[k] + sub * (S * H) + s - second * H * S) + second;
+        T* d = dst + 2 * ((int64_t)offsets[k] + i);
+        d[0] = p[0];
+        d[1] = p[2];
+    }
+}
+
+int table_samples(Table& t)
+{
+    static std::mutex mu;
+    std::lock_guard<std::mutex> lock(mu);
+    const dim3 grid(num_sms(), t.K);
+    const size_t n = std::max<int64_t>(t.n_samples, 1);
+    const bool f32 = !t.data, lp = t.store != WG_F32 && !t.data_lp;
+    if ((f32 && cudaMalloc(&t.data, sizeof(float2) * n) != cudaSuccess) || (lp && cudaMalloc(&t.data_lp, 4 * n) != cudaSuccess)) {
+        cudaGetLastError();
+        if (f32) {
+            cudaFree(t.data);
+            t.data = nullptr;
+        }
+        return fail(WG_E_OOM, "cannot allocate the table's samples in their order (%zu)", n);
+    }
+    if (f32) {
+        k_samples<<<grid, 256>>>(reinterpret_cast<const float*>(t.pairs), t.supports_d, t.offsets_d, t.poffsets_d, t.beta * t.beta,
+                                 reinterpret_cast<float*>(t.data));
+        WG_LAUNCHED("k_samples");
+    }
+    if (lp) {
+        k_samples<<<grid, 256>>>(static_cast<const unsigned short*>(t.pairs_lp), t.supports_d, t.offsets_d, t.poffsets_d,
+                                 t.beta * t.beta, static_cast<unsigned short*>(t.data_lp));
+        WG_LAUNCHED("k_samples");
+    }
+    if (f32 || lp) WG_CUDA(cudaDeviceSynchronize());
+    return WG_OK;
+}
+
+int table_to_host(const Table& t, float* data)
+{
+    std::vector<float4> h;
+    const int b2 = t.beta * t.beta;
+    int64_t poff = 0;
+    for (int k = 0; k < t.K; ++k) {
+        const int S = t.supports[k], H = (S + 1) / 2;
+        const int64_t n = (int64_t)b2 * S * H;
+        h.resize(n);
+        WG_CUDA(cudaMemcpy(h.data(), t.pairs + poff, sizeof(float4) * n, cudaMemcpyDeviceToHost));
+        float* d = data + 2 * (int64_t)t.offsets[k];
+        for (int sub = 0; sub < b2; ++sub)
+            for (int s = 0; s < S * S; ++s, d += 2) {
+                const float4 v = h[(int64_t)sub * S * H + (s < H * S ? s : s - H * S)];
+                d[0] = s < H * S ? v.x : v.y;
+                d[1] = s < H * S ? v.z : v.w;
+            }
+        poff += n;
+    }
+    return WG_OK;
 }
 
 int set_table_store(Table& t, int store)
@@ -201,17 +244,13 @@ int set_table_store(Table& t, int store)
     t.pairs_lp = nullptr;
     t.store = WG_F32;
     if (store == WG_F32) return WG_OK;
-    if (cudaMalloc(&t.data_lp, 4 * (size_t)std::max<int64_t>(t.n_samples, 1)) != cudaSuccess ||
-        cudaMalloc(&t.pairs_lp, 8 * (size_t)std::max<int64_t>(t.n_pairs, 1)) != cudaSuccess) {
+    if (cudaMalloc(&t.pairs_lp, 8 * (size_t)std::max<int64_t>(t.n_pairs, 1)) != cudaSuccess) {
         cudaGetLastError();
-        cudaFree(t.data_lp);
-        t.data_lp = nullptr;
         return fail(WG_E_OOM, "cannot allocate the low-precision table");
     }
     if (t.n_samples > 0) {
-        k_table_lp<<<(unsigned)((t.n_samples + 255) / 256), 256>>>(t.data, t.n_samples, store, t.data_lp);
-        WG_LAUNCHED("k_table_lp");
-        if (int rc = fill_pairs(t, store, t.pairs_lp, nullptr)) return rc;
+        k_pairs_lp<<<(unsigned)((t.n_pairs + 255) / 256), 256>>>(t.pairs, t.n_pairs, store, static_cast<uint2*>(t.pairs_lp));
+        WG_LAUNCHED("k_pairs_lp");
     }
     WG_CUDA(cudaDeviceSynchronize());
     t.store = store;
@@ -264,8 +303,7 @@ static int finish_layout(Table& t)
     const size_t K = t.K, nz = K * t.beta * t.beta;
     const size_t bytes = sizeof(double) * (nz + 2 * K) + sizeof(int) * 4 * K + sizeof(float) * nz;
     unsigned char* d = nullptr;
-    if (cudaMalloc(&t.data, sizeof(float2) * std::max<int64_t>(off, 1)) != cudaSuccess ||
-        cudaMalloc(&t.pairs, sizeof(float4) * std::max<int64_t>(poff, 1)) != cudaSuccess ||
+    if (cudaMalloc(&t.pairs, sizeof(float4) * std::max<int64_t>(poff, 1)) != cudaSuccess ||
         cudaMalloc(&d, bytes) != cudaSuccess) {
         cudaGetLastError();
         free_table(t);
@@ -393,13 +431,15 @@ int build_table(const wg_table_desc& d, Table& t, cudaStream_t s)
         if (rc != WG_OK) break;
         rc = finish_layout(t);
         if (rc != WG_OK) break;
+        int64_t poff = 0;
         for (int k = 0; k < K; ++k) {
             k_fill_plane<<<nb, 256, 0, s>>>(taper, n_k, M, d.du, wscreen[k], plane);
             count_launch();
             if (cufftExecZ2Z(plan, plane, plane, CUFFT_FORWARD) != CUFFT_SUCCESS) { rc = fail(WG_E_CUDA, "cufftExecZ2Z"); break; }
-            k_trim<<<beta * beta, 256, 0, s>>>(plane, M, beta, t.supports[k], norm, t.data + t.offsets[k],
+            k_trim<<<beta * beta, 256, 0, s>>>(plane, M, beta, t.supports[k], norm, t.pairs + poff,
                                                 t.zeta + (int64_t)k * beta * beta);
             count_launch();
+            poff += (int64_t)beta * beta * t.supports[k] * ((t.supports[k] + 1) / 2);
         }
         if (rc != WG_OK) break;
         {
@@ -407,7 +447,6 @@ int build_table(const wg_table_desc& d, Table& t, cudaStream_t s)
             k_zeta_f32<<<(nz + 255) / 256, 256, 0, s>>>(t.zeta, nz, t.zeta_f);
             count_launch();
         }
-        if ((rc = fill_pairs(t, WG_F32, t.pairs, s)) != WG_OK) break;
         cudaError_t e = cudaStreamSynchronize(s);
         if (e != cudaSuccess) rc = cuda_fail(e, "conv_table_build");
     } while (0);
@@ -435,20 +474,33 @@ int import_table(int K, int beta, double w_max, double du, int s0, const int* su
             return fail(WG_E_INVALID_ARG, "support %d of plane %d must be odd, in [1, %d]", t.supports[k], k, kMaxSupport);
     int rc = finish_layout(t);
     if (rc != WG_OK) return rc;
-    std::vector<float2> h((size_t)t.n_samples);
-    for (int64_t i = 0; i < t.n_samples; ++i) h[i] = make_float2((float)data[2 * i], (float)data[2 * i + 1]);
+    std::vector<float4> h((size_t)t.n_pairs, make_float4(0.f, 0.f, 0.f, 0.f));
+    {
+        float4* p = h.data();
+        for (int k = 0; k < K; ++k) {
+            const int S = t.supports[k], H = (S + 1) / 2;
+            for (int sub = 0; sub < beta * beta; ++sub, p += S * H, data += 2 * S * S)
+                for (int s = 0; s < S * S; ++s) {
+                    const float re = (float)data[2 * s], im = (float)data[2 * s + 1];
+                    if (s < H * S) {
+                        p[s].x = re;
+                        p[s].z = im;
+                    } else {
+                        p[s - H * S].y = re;
+                        p[s - H * S].w = im;
+                    }
+                }
+        }
+    }
     std::vector<float> zf((size_t)K * beta * beta);
     for (size_t i = 0; i < zf.size(); ++i) zf[i] = (float)zeta[i];
-    if (cudaMemcpy(t.data, h.data(), sizeof(float2) * h.size(), cudaMemcpyHostToDevice) != cudaSuccess ||
+    if (cudaMemcpy(t.pairs, h.data(), sizeof(float4) * h.size(), cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(t.zeta, zeta, sizeof(double) * K * beta * beta, cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(t.zeta_f, zf.data(), sizeof(float) * zf.size(), cudaMemcpyHostToDevice) != cudaSuccess) {
         free_table(t);
         return fail(WG_E_CUDA, "table upload failed");
     }
-    int rc2 = fill_pairs(t, WG_F32, t.pairs, nullptr);
-    if (rc2 == WG_OK && cudaDeviceSynchronize() != cudaSuccess) rc2 = cuda_fail(cudaGetLastError(), "k_table_pairs");
-    if (rc2 != WG_OK) free_table(t);
-    return rc2;
+    return WG_OK;
 }
 
 }  // namespace wg
