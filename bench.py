@@ -82,9 +82,8 @@ SYNTH_NAME = {"wstack_2k": ("wproj_2k", {"n_chan": 4})}
 CHAN_GROUP = {"batch_8k": 8}
 # gridder plans the autotuner tries (seg_len, slots, fixed R): on the batch for the single-grid
 # workloads, per channel group for the batched one
-STEP_PLANS = [(128, 256, False), (128, 256, True), (256, 256, True), (64, 256, True), (128, 128, True),
-              (128, 128, False)]
-BATCH_PLANS = [(256, 256, True), (256, 256, False), (128, 256, True), (256, 128, True)]
+STEP_PLANS = [(128, 256, False), (256, 256, False), (64, 256, False), (128, 128, False)]
+BATCH_PLANS = [(256, 256, False), (128, 256, False), (256, 128, False)]
 
 
 def _peaks():

@@ -371,7 +371,7 @@ int worklist_get_plan(const wg_worklist* wl, wg_plan* plan);
 
 /* Autotuner (not in the thesis; it picks the GPU work decomposition of the gridding phase,
  * Sec. 4.3.3).  Times grid_vis on the batch prepared on `wl` under each of the n_candidates plans (NULL or
- * 0: seg_len {64, 128, 256} x slots {128, 256} x flags {0, WG_PLAN_FIXED_R}), `repeats`
+ * 0: seg_len {64, 128, 256} x slots {128, 256}), `repeats`
  * timed launches each after one warm-up launch (CUDA events on `stream`), keeps the fastest
  * plan in `wl` and copies it to *best (may be NULL), writes its mean milliseconds per launch
  * to *best_ms (may be NULL), and then zeroes the grid (grid_zero: data, normaliser and

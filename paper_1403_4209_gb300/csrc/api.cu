@@ -550,8 +550,7 @@ int grid_autotune(wg_grid* gh, const wg_table* th, wg_worklist* wh, const wg_pla
         list.assign(cands, cands + n_cands);
     } else {
         for (int seg : {64, 128, 256})
-            for (int slots : {128, 256})
-                for (int flags : {0, WG_PLAN_FIXED_R}) list.push_back(wg_plan{seg, slots, flags, 0});
+            for (int slots : {128, 256}) list.push_back(wg_plan{seg, slots, 0, 0});      // (WG_PLAN_FIXED_R changes nothing)
     }
     for (const wg_plan& p : list)
         if (int rc = check_plan(p)) return rc;
