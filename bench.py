@@ -212,11 +212,22 @@ def measured_ceilings(real_rate: float, P: int) -> dict:
                     "(ncu l1tex hit rate about 8 %), so the fetch ceiling is the L2 one"}
 
 
+GRIDDER_SOURCES = ("grid.cu", "pairs.cuh", "internal.cuh")
+
+
+def _gridder_sources_hash():
+    """the gridder's source and the headers that hold the rest of it (staging, sample loads, tasks)"""
+    h = hashlib.sha256()
+    for name in GRIDDER_SOURCES:
+        with open(os.path.join(ROOT, "paper_1403_4209_gb300", "csrc", name), "rb") as f:
+            h.update(f.read())
+    return h.hexdigest()[:16]
+
+
 def _gridder_traffic(per_launch_units):
     """DRAM bytes per k_grid launch from the committed ncu summary, scaled to this launch's
-    gridded updates; None if the gridder source changed since the counters were taken."""
+    gridded updates; None if a gridder source changed since the counters were taken."""
     prof = os.path.join(ROOT, "profiles", "k_grid_wproj_2k.md")
-    src = os.path.join(ROOT, "paper_1403_4209_gb300", "csrc", "grid.cu")
     if not os.path.exists(prof):
         return None
     kv = {}
@@ -226,8 +237,7 @@ def _gridder_traffic(per_launch_units):
                 k, v = line[2:].rsplit(":", 1)
                 kv[k.strip()] = v.strip().strip("`")
     try:
-        h = hashlib.sha256(open(src, "rb").read()).hexdigest()[:16]
-        if kv.get("grid.cu sha256[:16]") != h:
+        if kv.get("gridder sources sha256[:16]") != _gridder_sources_hash():
             return None
         return float(kv["dram bytes per update"]) * per_launch_units
     except (KeyError, ValueError):
