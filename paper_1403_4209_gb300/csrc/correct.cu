@@ -21,11 +21,13 @@
 // What bounds it: HBM, and the transforms' own passes.  Measured (grid_correct): Stokes I of 16 channels of 2048^2 x 4
 // 1.93 -> 0.78 ms; of 4 channels of 8192^2 x 1 5.24 -> 2.29 ms; I, Q, U, V of 3 channels of 1500^2 569 -> 428 us; w-stacking of
 // 32 planes of 2048^2 x 1 3.72 -> 1.36 ms (32 launches that each read and wrote the sums, and FP64 phases, before).
-// WG_IMAGE_PER_POL_RAW skips the division by N_p.  It images the residuals of a fit to visibilities, and keeps complex
-// transforms: of these smooth, peaked grids cuFFT's complex-to-real ones came out less accurate at sides that are powers
-// of two (rel-L2 against 64 bits 3.1e-7 against 2.5e-7 at 1024^2, and 3.2e-7 against 2.5e-7 at 2048^2; the gradient of a fit at
-// 1024^2 4.4e-7 against 3.3e-7).  Of gridded observations they are as accurate (1024^2: 3.2e-7 against 3.1e-7) or more so
-// (512^2 2.2 against 2.6, 1500^2 2.5 against 2.9, 2048^2 2.7 against 3.1, 8192^2 3.3 against 3.6).  WG_IMAGE_TRANSPOSE applies the exact transpose
+// WG_IMAGE_PER_POL_RAW skips the division by N_p.  It images the residuals of a fit to visibilities, and at sides that are
+// powers of two it keeps complex transforms: of these smooth, peaked grids cuFFT's complex-to-real ones came out less
+// accurate there (rel-L2 against 64 bits 3.1e-7 against 2.5e-7 at 1024^2, and 3.2e-7 against 2.5e-7 at 2048^2; the gradient of a
+// fit at 1024^2 4.4e-7 against 3.4e-7), at other sides as accurate or more so (gradients 3.4e-7 against 4.1e-7 at 896^2, 3.6
+// against 3.8 at 1152^2, 2.6 against 2.8 at 1500^2).  Of gridded observations they are as accurate (1024^2: 3.2e-7 against
+// 3.1e-7) or more so (512^2 2.2 against 2.6, 1500^2 2.5 against 2.9, 2048^2 2.7 against 3.1, 8192^2 3.3 against 3.6).
+// WG_IMAGE_TRANSPOSE applies the exact transpose
 // of that map (the adjoint of Re(inverse FFT) under the real inner product is the forward FFT of
 // the real image): grid = (-1)^(x+y) FFT_forward((-1)^(mx+my) img / (taper sinc)), a real-to-complex
 // transform whose other half plane k_expand mirrors into the grid.
@@ -108,7 +110,7 @@ __global__ void __launch_bounds__(256) k_hermitian(const float2* __restrict__ gr
 {
     __shared__ float s_in[P];
     const int y = blockIdx.y, gch = blockIdx.z, G = gridDim.z, M = N / 2 + 1;
-    if (threadIdx.x < P) s_in[threadIdx.x] = inv_norm(norm[gch * P + threadIdx.x]);
+    if (threadIdx.x < P) s_in[threadIdx.x] = mode == WG_IMAGE_PER_POL_RAW ? 1.f : inv_norm(norm[gch * P + threadIdx.x]);
     __syncthreads();
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     if (x >= M) return;
@@ -200,7 +202,7 @@ __global__ void __launch_bounds__(256) k_planes(const float2* __restrict__ grid,
     for (int p = 0; p < P; ++p) f[(blockIdx.y * (int64_t)P + p) * nn + pix] = v[p];
 }
 
-// WG_IMAGE_PER_POL_RAW: the real parts of the planes f[gch][p][N][N] (blockIdx.z) of the inverse transforms (not
+// WG_IMAGE_PER_POL_RAW, N a power of two: the real parts of the planes f[gch][p][N][N] (blockIdx.z) of the inverse transforms (not
 // demodulated, so that pixel m is at (m + N/2) mod N) times (-1)^(mx+my) / (taper sinc)
 __global__ void __launch_bounds__(256) k_image_out(const float2* __restrict__ f, int N, const float* __restrict__ icorr,
                                                    float* __restrict__ img)
@@ -311,10 +313,11 @@ static int correct_impl(Grid& g, const Table& t, int mode, float* image, cudaStr
         g.scratch_chans = G;
     }
     const int G = g.scratch_chans;
+    const bool raw_c2c = mode == WG_IMAGE_PER_POL_RAW && (N & (N - 1)) == 0;
     {
         int rc;
         if (mode == WG_IMAGE_TRANSPOSE) rc = make_plan(g.plan_r2c, N, CUFFT_R2C, G * P);
-        else if (mode == WG_IMAGE_WSTACK || mode == WG_IMAGE_PER_POL_RAW) rc = make_plan(g.plan_c2c, N, CUFFT_C2C, G * P);
+        else if (mode == WG_IMAGE_WSTACK || raw_c2c) rc = make_plan(g.plan_c2c, N, CUFFT_C2C, G * P);
         else rc = make_plan(g.plan_c2r, N, CUFFT_C2R, G);
         if (rc != WG_OK) return rc;
     }
@@ -360,7 +363,7 @@ static int correct_impl(Grid& g, const Table& t, int mode, float* image, cudaStr
             return fail(WG_E_CUDA, "cufftExecC2C failed");
         return WG_OK;
     };
-    if (mode == WG_IMAGE_PER_POL_RAW) {
+    if (raw_c2c) {
         if (cufftSetStream(g.plan_c2c, s) != CUFFT_SUCCESS) return fail(WG_E_CUDA, "cufftSetStream failed");
         for (int c0 = 0; c0 < C; c0 += G) {
             if (int rc = transform(c0)) return rc;
@@ -395,7 +398,7 @@ static int correct_impl(Grid& g, const Table& t, int mode, float* image, cudaStr
         return rc;
     }
     const int no = mode == WG_IMAGE_STOKES_I ? 1 : P;
-    const bool scaled = mode == WG_IMAGE_PER_POL || P == 1;
+    const bool scaled = mode == WG_IMAGE_PER_POL || (P == 1 && mode != WG_IMAGE_PER_POL_RAW);
     if (cufftSetStream(g.plan_c2r, s) != CUFFT_SUCCESS) return fail(WG_E_CUDA, "cufftSetStream failed");
     float2* hp = g.scratch;                    // half planes [no][G], then the real planes behind them
     float* real = reinterpret_cast<float*>(g.scratch + ((size_t)no * G * N * M + 31) / 32 * 32);
