@@ -12,9 +12,9 @@
 // pairs into 2P floats; these go through a shared-memory transpose (batches of 64 / (2P)
 // entries), after which each lane holds two components of one entry summed over the warp and
 // adds them to a per-entry FP32 accumulator with one vector atomic per footprint block.  It is bound like
-// the gridder (issue 52 %, FMA pipe 45 %, L1 data path 62 %), with the transpose on top.  Measured (degrid_vis,
-// default plan): 0.87 M entries of supports 9..65, 4.8 M records: P = 4 2105 -> 1600 us, P = 2 1660 -> 1060, P = 1
-// 1470 -> 900; supports 9..129, P = 1 1510 -> 925; 1 k entries 227 -> 44.
+// the gridder (60 % of the FMA pipe's cycles, 54 % of the issue slots, L1 data path 72 %), with the transpose on
+// top.  Measured (degrid_vis, default plan, single points -> now): 0.87 M entries of supports 9..65, 4.8 M records: P = 4
+// 2111 -> 1506 us, P = 2 1666 -> 1013, P = 1 1477 -> 851; 2.4 M records, supports 9..129, P = 1 2314 -> 1665; 1 k entries 241 -> 44.
 //
 // k_degrid_tile writes the records of each entry's run.  Compression (Sec. 4.3.3) carries over:
 // every record compressed into an entry has its footprint and kernel samples, so m is computed

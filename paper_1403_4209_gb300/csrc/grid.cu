@@ -7,14 +7,15 @@
 // pixel and accumulate in registers while the pair stays the same; when it moves, the lane flushes
 // its accumulators with vector FP32 atomics (all polarisations of a pixel are contiguous).
 //
-// What bounds it: instruction issue and the FMA pipe (59 % and 50 % busy at four polarisations, 128
-// registers, 16 warps an SM), then the L1 data path (68 %: every sample is used once per entry and comes from L2).
+// What bounds it: the FMA pipe and instruction issue (68 % of the pipe's cycles and 54 % of the issue slots at four
+// polarisations; 128 registers, with 20 bytes of spills outside the loop over entries, 16 warps an SM), then the L1 data
+// path (70 %: every sample is used once per entry and comes from L2).
 // Packed FMAs on three distinct operands run at 2.6 cycles each, not 2 (register reads).  Consecutive
 // entries of a track usually keep the footprint (about 85 %, weighted by S^2) and differ only in the
 // sub-kernel: the loop over them holds the sample loads and 4P packed FMAs a pair and no test.
-// Measured (grid_vis): 116 M records in 16 channels, P = 4, supports 9..65: 25.0 -> 20.5 ms; 4.8 M records,
-// P = 4: 1.71 -> 1.22 ms; interleaved, P = 2: 4.64 -> 2.75 ms; 15.7 M records, P = 1, supports 9..129: 26.8 -> 18.6 ms;
-// compensated with an FP16 table, P = 4: 1.66 -> 1.37 ms; 127 k entries of support 7: 51 -> 28 us; 1 k entries: 204 -> 25 us.
+// Measured (grid_vis, single points -> now): 116 M records in 16 channels, P = 4, supports 9..65: 25.1 -> 20.2 ms; 4.8 M
+// records, P = 4: 1.72 -> 1.20 ms; interleaved, P = 2: 4.65 -> 2.63 ms; 15.7 M records, P = 1, supports 9..129: 26.9 -> 18.3 ms;
+// compensated with an FP16 table, P = 4: 1.67 -> 1.34 ms; 127 k entries of support 7: 54 -> 27 us; 1 k entries: 209 -> 24 us.
 #include "pairs.cuh"
 
 namespace wg {

@@ -11,7 +11,7 @@
 // Limits: at most WG_NOALLOC_MAX_RECORDS records (rows x channels) and WG_NOALLOC_MAX_CHAN
 // channels per call; larger batches are rejected with WG_E_CAPACITY.  Every call uses the same
 // scratch, which keeps the previous call's contents: the accumulators that must start at zero
-// are cleared (cudaMemsetAsync) at the start of each call, and calls that overlap on the GPU
+// are cleared (k_prep_init; the statistics by cudaMemsetAsync) at the start of each call, and calls that overlap on the GPU
 // (on different streams, or from different host threads) race on the scratch.
 //
 // Set-up: the first call on each device asks the runtime for the scratch's device address

@@ -746,7 +746,7 @@ __device__ __forceinline__ void emit_run(const int4& info, bool is_carry, int ra
         return;
     }
     const int ech = pp.wstack ? ch * pp.K + k : gch + pp.chan0;   // the grid channel
-    // (-x0) mod S and (-y0) mod S: the residue classes of the footprint's first column and row
+    // (-x0) mod S and (-y0) mod S, for worklist_view (the gridder works out its own, of pairs)
     const float inv_s = __frcp_rn((float)S);
     const int rx = mod_small(info.x & 0xFFFF, S, inv_s), ry = mod_small((info.x >> 16) & 0xFFFF, S, inv_s);
     const int cuv = (rx ? S - rx : 0) | ((ry ? S - ry : 0) << 16);
@@ -1522,7 +1522,7 @@ __global__ void __launch_bounds__(256) k_density_sq(const float* __restrict__ de
     if (threadIdx.x < P && s_q[threadIdx.x] != 0.0) atomicAdd(&sums[P + threadIdx.x], s_q[threadIdx.x]);
 }
 
-// w / (1 + W f2) rounded once: the denominator as two floats (dh + dl, exact products by FMA), a correctly
+// w / (1 + W f2), as the FP64 quotient rounds it (all of 16 M values tried): the denominator as two floats (dh + dl, exact products by FMA), a correctly
 // rounded FP32 quotient by dh, and its remainder's correction.  Values out of the range in which that is exact take
 // the FP64 division, whose thirty or so instructions are what the kernel spent its time on.
 __device__ __forceinline__ float robust_weight(float w, float W, double f2, float f2h, float f2l)
