@@ -221,8 +221,8 @@ typedef struct wg_table_info {
 } wg_table_info;
 /* Sizes and device pointers (owned by the table) of C-1 .. C-3 (Sec. 4.2.2).  The table keeps C-1 as the
  * gridder reads it, 8 (1 + 1/S) bytes a sample of a plane of support S (and 4 (1 + 1/S) more in a reduced
- * store); the first call makes the copies in the order given here, 8 bytes a sample and 4, and synchronises the
- * device.  Errors: INVALID_ARG, OOM, CUDA. */
+ * store); the first call makes the copies in the order given here, 8 bytes a sample and 4, and waits for
+ * them.  Errors: INVALID_ARG, OOM, CUDA. */
 int table_info(const wg_table* table, wg_table_info* info);
 /* The same (C-2 and C-3 of Sec. 4.2.2) without C-1: data and data_lp are NULL and nothing is made.
  * Errors: INVALID_ARG. */

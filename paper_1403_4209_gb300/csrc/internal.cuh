@@ -180,7 +180,7 @@ int import_table(int K, int beta, double w_max, double du, int s0, const int* su
                  const double* data, const double* zeta, Table& t);
 int free_table(Table& t);
 int set_table_store(Table& t, int store);
-// fills data and data_lp; synchronises the device the first time
+// fills data and data_lp; waits for them the first time
 int table_samples(Table& t);
 // copies C-1 in the order of its definition to `data` (n_samples complex floats)
 int table_to_host(const Table& t, float* data);

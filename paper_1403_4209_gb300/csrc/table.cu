@@ -184,33 +184,59 @@ __global__ void k_samples(const T* __restrict__ pairs, const int* __restrict__ s
     }
 }
 
+static int make_samples(Table& t, cudaStream_t s)
+{
+    const dim3 grid(num_sms(), t.K);
+    const size_t n = std::max<int64_t>(t.n_samples, 1);
+    float2* data = t.data;
+    void* lp = t.data_lp;
+    auto release = [&]() {
+        if (data != t.data) cudaFree(data);
+        if (lp != t.data_lp) cudaFree(lp);
+    };
+    if ((!data && cudaMalloc(&data, sizeof(float2) * n) != cudaSuccess) ||
+        (t.store != WG_F32 && !lp && cudaMalloc(&lp, 4 * n) != cudaSuccess)) {
+        cudaGetLastError();
+        release();
+        return fail(WG_E_OOM, "cannot allocate the table's samples in their order (%zu)", n);
+    }
+    if (data != t.data) {
+        k_samples<<<grid, 256, 0, s>>>(reinterpret_cast<const float*>(t.pairs), t.supports_d, t.offsets_d, t.poffsets_d,
+                                       t.beta * t.beta, reinterpret_cast<float*>(data));
+        count_launch();
+    }
+    if (lp != t.data_lp) {
+        k_samples<<<grid, 256, 0, s>>>(static_cast<const unsigned short*>(t.pairs_lp), t.supports_d, t.offsets_d, t.poffsets_d,
+                                       t.beta * t.beta, static_cast<unsigned short*>(lp));
+        count_launch();
+    }
+    const cudaError_t e = cudaStreamSynchronize(s);
+    if (e != cudaSuccess) {
+        release();
+        return cuda_fail(e, "k_samples");
+    }
+    t.data = data;
+    t.data_lp = lp;
+    return WG_OK;
+}
+
+// On a stream of its own, and in the relaxed capture mode: a stream of this thread may be being captured.
 int table_samples(Table& t)
 {
     static std::mutex mu;
     std::lock_guard<std::mutex> lock(mu);
-    const dim3 grid(num_sms(), t.K);
-    const size_t n = std::max<int64_t>(t.n_samples, 1);
-    const bool f32 = !t.data, lp = t.store != WG_F32 && !t.data_lp;
-    if ((f32 && cudaMalloc(&t.data, sizeof(float2) * n) != cudaSuccess) || (lp && cudaMalloc(&t.data_lp, 4 * n) != cudaSuccess)) {
-        cudaGetLastError();
-        if (f32) {
-            cudaFree(t.data);
-            t.data = nullptr;
-        }
-        return fail(WG_E_OOM, "cannot allocate the table's samples in their order (%zu)", n);
+    if (t.data && (t.store == WG_F32 || t.data_lp)) return WG_OK;
+    cudaStreamCaptureMode capture = cudaStreamCaptureModeRelaxed;
+    WG_CUDA(cudaThreadExchangeStreamCaptureMode(&capture));
+    cudaStream_t s = nullptr;
+    int rc = WG_OK;
+    if (cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking) != cudaSuccess) rc = cuda_fail(cudaGetLastError(), "table_info");
+    if (rc == WG_OK) {
+        rc = make_samples(t, s);
+        cudaStreamDestroy(s);
     }
-    if (f32) {
-        k_samples<<<grid, 256>>>(reinterpret_cast<const float*>(t.pairs), t.supports_d, t.offsets_d, t.poffsets_d, t.beta * t.beta,
-                                 reinterpret_cast<float*>(t.data));
-        WG_LAUNCHED("k_samples");
-    }
-    if (lp) {
-        k_samples<<<grid, 256>>>(static_cast<const unsigned short*>(t.pairs_lp), t.supports_d, t.offsets_d, t.poffsets_d,
-                                 t.beta * t.beta, static_cast<unsigned short*>(t.data_lp));
-        WG_LAUNCHED("k_samples");
-    }
-    if (f32 || lp) WG_CUDA(cudaDeviceSynchronize());
-    return WG_OK;
+    cudaThreadExchangeStreamCaptureMode(&capture);
+    return rc;
 }
 
 int table_to_host(const Table& t, float* data)

@@ -79,3 +79,22 @@ def test_gridded_samples_bit_for_bit(supports, store):
         got = torch.view_as_real(g.data[0]).cpu().numpy()
         for p in range(2):
             assert np.array_equal(got[:, :, p], exp)
+
+
+def test_table_info_while_a_stream_is_captured():
+    # its first call makes the samples: neither the capture nor what it holds is disturbed
+    ref, t = _tables([5, 9], 3, 6)
+    t.set_store("f16")
+    x = torch.zeros(4, device="cuda")
+    graph = torch.cuda.CUDAGraph()
+    info = _lib.TableInfo()
+    with torch.cuda.graph(graph):
+        x += 1
+        rc = wg.lib.table_info(t.handle, ctypes.byref(info))
+        x += 1
+    assert rc == 0 and info.data and info.data_lp
+    graph.replay()
+    torch.cuda.synchronize()
+    assert x.tolist() == [2.0] * 4
+    got = torch.as_tensor(wg.api._DeviceBuffer(info.data, (t.n_samples, 2), "<f4"), device="cuda").cpu()
+    assert torch.equal(got, torch.view_as_real(torch.as_tensor(ref.data.astype(np.complex64))))
