@@ -16,7 +16,9 @@
 //   6. zeta = sum of real parts of each sub-kernel (eq. "sum"), in FP64 before rounding to FP32.
 #include <cmath>
 #include <cstdio>
+#include <memory>
 #include <mutex>
+#include <new>
 #include <vector>
 
 #include <cuda_bf16.h>
@@ -186,7 +188,7 @@ __global__ void k_samples(const T* __restrict__ pairs, const int* __restrict__ s
 
 static int make_samples(Table& t, cudaStream_t s)
 {
-    const dim3 grid(num_sms(), t.K);
+    const dim3 grid(num_sms() * 8, t.K);
     const size_t n = std::max<int64_t>(t.n_samples, 1);
     float2* data = t.data;
     void* lp = t.data_lp;
@@ -241,8 +243,19 @@ int table_samples(Table& t)
 
 int table_to_host(const Table& t, float* data)
 {
-    std::vector<float4> h;
     const int b2 = t.beta * t.beta;
+    // put in order on the device and copied at once if there is room, otherwise plane by plane and put in order here
+    float2* tmp = nullptr;
+    if (cudaMalloc(&tmp, sizeof(float2) * (size_t)std::max<int64_t>(t.n_samples, 1)) == cudaSuccess) {
+        k_samples<<<dim3(num_sms() * 8, t.K), 256>>>(reinterpret_cast<const float*>(t.pairs), t.supports_d, t.offsets_d, t.poffsets_d,
+                                                     b2, reinterpret_cast<float*>(tmp));
+        count_launch();
+        const cudaError_t e = cudaMemcpy(data, tmp, sizeof(float2) * (size_t)t.n_samples, cudaMemcpyDeviceToHost);
+        cudaFree(tmp);
+        return e == cudaSuccess ? WG_OK : cuda_fail(e, "table_copy_to_host");
+    }
+    cudaGetLastError();
+    std::vector<float4> h;
     int64_t poff = 0;
     for (int k = 0; k < t.K; ++k) {
         const int S = t.supports[k], H = (S + 1) / 2;
@@ -250,12 +263,17 @@ int table_to_host(const Table& t, float* data)
         h.resize(n);
         WG_CUDA(cudaMemcpy(h.data(), t.pairs + poff, sizeof(float4) * n, cudaMemcpyDeviceToHost));
         float* d = data + 2 * (int64_t)t.offsets[k];
-        for (int sub = 0; sub < b2; ++sub)
-            for (int s = 0; s < S * S; ++s, d += 2) {
-                const float4 v = h[(int64_t)sub * S * H + (s < H * S ? s : s - H * S)];
-                d[0] = s < H * S ? v.x : v.y;
-                d[1] = s < H * S ? v.z : v.w;
+        for (int sub = 0; sub < b2; ++sub) {
+            const float4* q = h.data() + (int64_t)sub * S * H;
+            for (int i = 0; i < S * H; ++i, d += 2) {
+                d[0] = q[i].x;
+                d[1] = q[i].z;
             }
+            for (int i = 0; i < S * S - S * H; ++i, d += 2) {
+                d[0] = q[i].y;
+                d[1] = q[i].w;
+            }
+        }
         poff += n;
     }
     return WG_OK;
@@ -500,27 +518,24 @@ int import_table(int K, int beta, double w_max, double du, int s0, const int* su
             return fail(WG_E_INVALID_ARG, "support %d of plane %d must be odd, in [1, %d]", t.supports[k], k, kMaxSupport);
     int rc = finish_layout(t);
     if (rc != WG_OK) return rc;
-    std::vector<float4> h((size_t)t.n_pairs, make_float4(0.f, 0.f, 0.f, 0.f));
-    {
-        float4* p = h.data();
-        for (int k = 0; k < K; ++k) {
-            const int S = t.supports[k], H = (S + 1) / 2;
-            for (int sub = 0; sub < beta * beta; ++sub, p += S * H, data += 2 * S * S)
-                for (int s = 0; s < S * S; ++s) {
-                    const float re = (float)data[2 * s], im = (float)data[2 * s + 1];
-                    if (s < H * S) {
-                        p[s].x = re;
-                        p[s].z = im;
-                    } else {
-                        p[s - H * S].y = re;
-                        p[s - H * S].w = im;
-                    }
-                }
+    std::unique_ptr<float4[]> h(new (std::nothrow) float4[(size_t)t.n_pairs]);
+    if (!h) {
+        free_table(t);
+        return fail(WG_E_OOM, "host allocation failed");
+    }
+    float4* p = h.get();
+    for (int k = 0; k < K; ++k) {
+        const int S = t.supports[k], n = S * ((S + 1) / 2), both = S * S - n;
+        for (int sub = 0; sub < beta * beta; ++sub, p += n, data += 2 * S * S) {
+            const double* q = data + 2 * n;              // the samples of the second rows
+            for (int i = 0; i < both; ++i)
+                p[i] = make_float4((float)data[2 * i], (float)q[2 * i], (float)data[2 * i + 1], (float)q[2 * i + 1]);
+            for (int i = both; i < n; ++i) p[i] = make_float4((float)data[2 * i], 0.f, (float)data[2 * i + 1], 0.f);
         }
     }
     std::vector<float> zf((size_t)K * beta * beta);
     for (size_t i = 0; i < zf.size(); ++i) zf[i] = (float)zeta[i];
-    if (cudaMemcpy(t.pairs, h.data(), sizeof(float4) * h.size(), cudaMemcpyHostToDevice) != cudaSuccess ||
+    if (cudaMemcpy(t.pairs, h.get(), sizeof(float4) * (size_t)t.n_pairs, cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(t.zeta, zeta, sizeof(double) * K * beta * beta, cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(t.zeta_f, zf.data(), sizeof(float) * zf.size(), cudaMemcpyHostToDevice) != cudaSuccess) {
         free_table(t);
